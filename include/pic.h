@@ -78,7 +78,8 @@ typedef struct {
                                stages (0 = default: 8x8x8 in 3D, 16x16 in 2D) */
     int halo;               /* drift guard in cells around a tile (0..2; -1 = default 1) */
     int sort_interval;      /* sort the particles by tile every K steps (>= 1; 0 = default 10) */
-    int particles_per_block;/* particles per thread block work item (0 = default 8192) */
+    int particles_per_block;/* most particles a thread block's work item takes (0 = default 8192); the
+                               items of a small pool are shorter, so that every SM has one */
     double rho_bg;          /* uniform immobile background charge density (enters rho only) */
     void *cuda_stream;      /* cudaStream_t to enqueue on; NULL = the legacy default stream */
     int sort_order;         /* PIC_SORT_AUTO (0, default), PIC_SORT_STABLE, PIC_SORT_BANKED or

@@ -278,6 +278,27 @@ void graph_drop(pic_grid *g)
     g->graph_valid = false;
 }
 
+// Particles per work item of a pool of `total`: the grid's particles_per_block
+// (the limit the fixed-point scales are set for), or less when a small pool's
+// items would leave SMs idle.  The 2D FP64 run of 32x32 cells and 8192 particles
+// has 16 tiles: whole, they keep 16 of the 152 SMs busy for 85 us a step; in 128
+// items of 64 particles the step takes 51 us instead of 101.  FP64 takes four items
+// per SM (one block alone leaves the FP64 pipe idle while it stages and flushes
+// its tile) of at least 64 particles (a warp's FP64 instruction takes 16 cycles,
+// so two warps hide most latencies); FP32 one per SM of at least one round of the
+// block: 256x256 cells and 2^20 particles take 2.75 ms per 40 steps in 256 whole
+// tiles and 2.78 ms in 768 parts.
+int item_length(const pic_grid *g, long long total)
+{
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const long long slots = (long long)std::max(1, sms) * (g->prec == PIC_FP64 ? 4 : 1);
+    const long long least = std::min(g->ppi, g->prec == PIC_FP64 ? 64 : kThreads);
+    const long long len = (((total + slots - 1) / slots) + 31) & ~31LL;
+    return (int)std::max(least, std::min<long long>(len, g->ppi));
+}
+
 // (Re)allocate everything whose size depends on the particle count.
 int size_particle_buffers(pic_grid *g, long long total)
 {
@@ -305,7 +326,8 @@ int size_particle_buffers(pic_grid *g, long long total)
     g->sort.sums_capacity = sums;
     CK(dalloc(&g->tile_start, (size_t)g->total_tiles + 1), "tile starts");
     CK(dalloc(&g->item_scan, (size_t)g->total_tiles + 1), "item scan");
-    g->max_items = g->total_tiles + (int)((total + g->ppi - 1) / g->ppi) + 1;
+    g->item_len = item_length(g, total);
+    g->max_items = g->total_tiles + (int)((total + g->item_len - 1) / g->item_len) + 1;
     CK(dalloc(&g->items, (size_t)g->max_items), "work items");
     if (g->sort_order == PIC_SORT_CELL_LANES) {
         CK(dalloc(&g->lane_cell, (size_t)std::max(1, g->total_tiles) * 128), "lane cells");
@@ -417,7 +439,7 @@ int do_sort(pic_grid *g, bool defer = false)
     const unsigned *perm = nullptr;
     cudaError_t e = sort_and_build_items(g->prec, g->dims, g->stream, g->total, g->pool, g->pool_alt, g->d_groups,
                                          g->d_group_base, (int)g->groups.size(), g->d_runs, g->total_tiles, g->sort,
-                                         g->tile_start, g->item_scan, g->items, g->n_items, g->ppi,
+                                         g->tile_start, g->item_scan, g->items, g->n_items, g->item_len,
                                          g->halo + (g->order2 == 5 ? 1 : 0),   // the current tile's bank base
                                          g->sort_order == PIC_SORT_BANKED ? 1 : 0, g->order2 == 5 ? 1 : 0, &nl,
                                          g->sort_order == PIC_SORT_CELL_LANES ? g->lane_cell : nullptr,
@@ -1676,7 +1698,7 @@ static int restore_body(pic_grid *g, const void *src, int on_device, const State
     // starts give the work items back, and the sort schedule continues
     if (g->total > 0 && !g->groups.empty()) {
         int nl = 0;
-        cudaError_t e = build_items(g->stream, g->tile_start, g->total_tiles, g->ppi, g->d_groups,
+        cudaError_t e = build_items(g->stream, g->tile_start, g->total_tiles, g->item_len, g->d_groups,
                                     (int)g->groups.size(), g->sort, g->item_scan, g->items, g->n_items, &nl);
         launch_count_add(g, nl);
         if (e != cudaSuccess) return cuda_fail(e, "work items");

@@ -195,6 +195,7 @@ cudaError_t adjoint_set_smem_limit(int dims, int prec, size_t bytes);
 struct pic_grid {
     int dims = 3, prec = 0;
     int halo = 1, sort_interval = 10, ppi = 8192, sort_order = 0;   // sort_order: the resolved PIC_SORT_*
+    int item_len = 8192;     // particles per work item (<= ppi; item_length)
     int tile[3] = {8, 8, 8};
     int pitch[2] = {0, 0};   // x, y pitch of the shared tiles (chosen at create)
     cudaStream_t stream = nullptr;

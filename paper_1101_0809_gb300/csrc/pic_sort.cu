@@ -1085,6 +1085,9 @@ __global__ void k_items(const long long *tile_start, const unsigned *scan, int t
     if (t >= total_tiles) return;
     const long long b = tile_start[t], e = tile_start[t + 1];
     const int cnt = (int)((e - b + ppi - 1) / ppi);
+    // equal parts, in whole warps: part <= ppi (a multiple of 32), so that
+    // part * (cnt - 1) <= ppi * (cnt - 1) < e - b and no item is empty
+    const int part = cnt > 0 ? (int)((((e - b + cnt - 1) / cnt) + 31) & ~31LL) : ppi;
     int lo = 0, hi = ngroups;
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
@@ -1095,8 +1098,8 @@ __global__ void k_items(const long long *tile_start, const unsigned *scan, int t
         WorkItem w;
         w.group = lo;
         w.tile = t - groups[lo].tile_base;
-        w.begin = b + (long long)q * ppi;
-        w.end = w.begin + ppi < e ? w.begin + ppi : e;
+        w.begin = b + (long long)q * part;
+        w.end = w.begin + part < e ? w.begin + part : e;
         items[s + q] = w;
     }
     if (t == total_tiles - 1) *n_items = (int)(s + cnt);
