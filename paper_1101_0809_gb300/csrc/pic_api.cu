@@ -485,7 +485,8 @@ int launch_part(pic_grid *g, int mode)
     // after a deferred sort: read the old order through the permutation, write the new one
     cudaError_t e = launch_particles(g->dims, g->prec, mode, g->stream, g->items, g->n_items, g->max_items, g->d_runs,
                                      g->d_groups, perm ? g->pool_alt : g->pool, g->E, g->B, g->J, g->old_cell,
-                                     g->old_off, g->halo, g->tile[0], g->tile[1], g->tile[2], g->d_err, g->pitch[0],
+                                     g->old_off, g->halo, g->tile[0], g->tile[1], g->tile[2], g->d_err,
+                                     g->sort.keys[0], g->pitch[0],
                                      g->pitch[1], g->order2, perm ? &g->pool : nullptr, perm);
     launch_count_add(g, g->max_items > 0 ? 1 : 0);
     if (perm) {
@@ -1342,7 +1343,7 @@ static int persistent_step(pic_grid *g)
     const unsigned *perm = g->pending_perm;
     cudaError_t e = launch_step_persistent(g->dims, g->prec, g->stream, g->items, g->n_items, g->d_runs, g->d_groups,
                                            perm ? g->pool_alt : g->pool, g->E, g->B, g->J, g->halo, g->tile[0],
-                                           g->tile[1], g->tile[2], g->d_err, (int)g->runs.size(),
+                                           g->tile[1], g->tile[2], g->d_err, g->sort.keys[0], (int)g->runs.size(),
                                            g->d_run_cell_base, &g->persist_blocks, 1, g->pitch[0], g->pitch[1],
                                            g->d_ant_n, g->antennas, perm ? &g->pool : nullptr, perm);
     launch_count_add(g, 1);
@@ -1379,7 +1380,7 @@ static int capture_graph(pic_grid *g)
     if (g->persist_blocks <= 0) {
         cudaError_t ep = launch_step_persistent(g->dims, g->prec, g->stream, g->items, g->n_items, g->d_runs,
                                                 g->d_groups, g->pool, g->E, g->B, g->J, g->halo, g->tile[0],
-                                                g->tile[1], g->tile[2], g->d_err, (int)g->runs.size(),
+                                                g->tile[1], g->tile[2], g->d_err, g->sort.keys[0], (int)g->runs.size(),
                                                 g->d_run_cell_base, &g->persist_blocks, 0, g->pitch[0], g->pitch[1],
                                                 g->d_ant_n, g->antennas);
         if (ep != cudaSuccess) return cuda_fail(ep, "persistent kernel set-up");

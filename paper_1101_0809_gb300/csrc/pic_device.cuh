@@ -82,6 +82,7 @@ struct WorkItem {
     int group;
     int tile;             // tile index inside the run
     long long begin, end; // particle range of this item
+    int drifted;          // particles found past the staged tile, summed over the steps since the sort
 };
 
 template <typename R>

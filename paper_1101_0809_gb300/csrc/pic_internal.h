@@ -38,25 +38,26 @@ struct PoolBuf {
 
 // Launch helpers implemented in the .cu files.  All enqueue on `st` and return
 // a cudaError_t from the launch.
-cudaError_t launch_particles(int dims, int prec, int mode, cudaStream_t st, const WorkItem *items,
+cudaError_t launch_particles(int dims, int prec, int mode, cudaStream_t st, WorkItem *items,
                              const int *n_items, int max_items, const RunDev *runs, const GroupDev *groups,
                              const PoolBuf &P, void *const E[3], void *const B[3], void *const J[3],
                              int *old_cell, void *const old_off[3], int halo, int max_tile_x,
-                             int max_tile_y, int max_tile_z, int *err, int p0, int p1, int order2 = 3,
+                             int max_tile_y, int max_tile_z, int *err, unsigned *far_list, int p0, int p1, int order2 = 3,
                              const PoolBuf *src = nullptr, const unsigned *perm = nullptr);
 // With perm (mode 0, l_a = 1 1/2): the pool was just sorted but not yet
 // permuted; particle p of the new order is read from src at perm[p] and
 // written, stepped, to P.
+// far_list: pool-sized scratch of the launch (process_item).
 // order2 = 3: l_a = 1 1/2; 5: l_a = 2 1/2 (tiles one cell wider on every side).
 size_t particles_smem_bytes(int dims, int prec, int mode, int tx, int ty, int tz, int halo, int p0, int p1,
                             int order2 = 3);
 // One cooperative launch per step over every run (see k_step_persistent);
 // *grid_blocks = 0 asks for the occupancy-derived grid and returns it; launch = 0
 // only prepares (attributes and grid size), which must happen outside a capture.
-cudaError_t launch_step_persistent(int dims, int prec, cudaStream_t st, const WorkItem *items, const int *n_items,
+cudaError_t launch_step_persistent(int dims, int prec, cudaStream_t st, WorkItem *items, const int *n_items,
                                    const RunDev *runs, const GroupDev *groups, const PoolBuf &P, void *const E[3],
                                    void *const B[3], void *const J[3], int halo, int tx, int ty, int tz, int *err,
-                                   int nruns, const long long *run_cell_base, int *grid_blocks, int launch, int p0,
+                                   unsigned *far_list, int nruns, const long long *run_cell_base, int *grid_blocks, int launch, int p0,
                                    int p1, long long *ant_n, int antennas, const PoolBuf *src = nullptr,
                                    const unsigned *perm = nullptr);
 cudaError_t particles_set_smem_limit(int dims, int prec, int mode, size_t bytes, int order2 = 3);

@@ -40,8 +40,8 @@ static cudaError_t set_limit_t(int mode, size_t bytes)
     const int b = (int)bytes;
     switch (mode) {
     case 0: return set_limit_fused<DIM, R, GeoDyn>(b);
-    case 1: return cudaFuncSetAttribute(k_particles<DIM, R, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-    default: return cudaFuncSetAttribute(k_particles<DIM, R, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+    case 1: return set_limit_one<DIM, R, 1, GeoDyn>(b);
+    default: return set_limit_one<DIM, R, 2, GeoDyn>(b);
     }
 }
 
@@ -58,12 +58,12 @@ cudaError_t particles_set_smem_limit(int dims, int prec, int mode, size_t bytes,
 }
 
 
-cudaError_t launch_particles(int dims, int prec, int mode, cudaStream_t st, const WorkItem *items,
+cudaError_t launch_particles(int dims, int prec, int mode, cudaStream_t st, WorkItem *items,
                              const int *n_items, int max_items, const RunDev *runs, const GroupDev *groups,
                              const PoolBuf &P, void *const E[3], void *const B[3], void *const J[3],
                              int *old_cell, void *const old_off[3], int halo, int max_tile_x, int max_tile_y,
-                             int max_tile_z, int *err, int p0, int p1, int order2, const PoolBuf *src,
-                             const unsigned *perm)
+                             int max_tile_z, int *err, unsigned *far_list, int p0, int p1, int order2,
+                             const PoolBuf *src, const unsigned *perm)
 {
     if (perm && (mode != 0 || order2 != 3)) return cudaErrorInvalidValue;   // read through perm: fused l_a = 1 1/2 only
     const size_t smem =
@@ -71,17 +71,19 @@ cudaError_t launch_particles(int dims, int prec, int mode, cudaStream_t st, cons
     if (order2 == 5) {
         const int tile[3] = {max_tile_x, max_tile_y, max_tile_z};
         return launch_particles_o5(dims, prec, mode, st, max_items, smem, items, n_items, runs, groups, P, E, B, J,
-                                   old_cell, old_off, halo, err, tile, p0, p1);
+                                   old_cell, old_off, halo, err, far_list, tile, p0, p1);
     }
     if (order2 == 4)
         return launch_particles_w1(dims, prec, mode, st, max_items, smem, items, n_items, runs, groups, P, E, B, J,
-                                   old_cell, old_off, halo, err);
+                                   old_cell, old_off, halo, err, far_list);
     if (prec == 0) {
-        auto a = make_args<double>(items, n_items, runs, groups, P, E, B, J, old_cell, old_off, halo, err, src, perm);
+        auto a = make_args<double>(items, n_items, runs, groups, P, E, B, J, old_cell, old_off, halo, err, far_list, src,
+                                    perm);
         return dims == 3 ? launch_mode<3, double>(mode, st, max_items, smem, a)
                          : launch_mode<2, double>(mode, st, max_items, smem, a);
     }
-    auto a = make_args<float>(items, n_items, runs, groups, P, E, B, J, old_cell, old_off, halo, err, src, perm);
+    auto a = make_args<float>(items, n_items, runs, groups, P, E, B, J, old_cell, old_off, halo, err, far_list, src,
+                                    perm);
     if (mode == 0) {
         const int tile[3] = {max_tile_x, max_tile_y, max_tile_z};
         cudaError_t e = cudaSuccess;
@@ -91,20 +93,20 @@ cudaError_t launch_particles(int dims, int prec, int mode, cudaStream_t st, cons
                      : launch_mode<2, float>(mode, st, max_items, smem, a);
 }
 
-cudaError_t launch_step_persistent(int dims, int prec, cudaStream_t st, const WorkItem *items, const int *n_items,
+cudaError_t launch_step_persistent(int dims, int prec, cudaStream_t st, WorkItem *items, const int *n_items,
                                    const RunDev *runs, const GroupDev *groups, const PoolBuf &P, void *const E[3],
                                    void *const B[3], void *const J[3], int halo, int tx, int ty, int tz, int *err,
-                                   int nruns, const long long *run_cell_base, int *grid_blocks, int launch, int p0,
+                                   unsigned *far_list, int nruns, const long long *run_cell_base, int *grid_blocks, int launch, int p0,
                                    int p1, long long *ant_n, int antennas, const PoolBuf *src, const unsigned *perm)
 {
     void *none[3] = {nullptr, nullptr, nullptr};
     const size_t smem = particles_smem_bytes(dims, prec, 0, tx, ty, tz, halo, p0, p1);
     if (prec == 0) {
-        auto a = make_args<double>(items, n_items, runs, groups, P, E, B, J, nullptr, none, halo, err, src, perm);
+        auto a = make_args<double>(items, n_items, runs, groups, P, E, B, J, nullptr, none, halo, err, far_list, src, perm);
         return dims == 3 ? persistent_t<3, double>(st, smem, nruns, run_cell_base, a, grid_blocks, launch, ant_n, antennas)
                          : persistent_t<2, double>(st, smem, nruns, run_cell_base, a, grid_blocks, launch, ant_n, antennas);
     }
-    auto a = make_args<float>(items, n_items, runs, groups, P, E, B, J, nullptr, none, halo, err, src, perm);
+    auto a = make_args<float>(items, n_items, runs, groups, P, E, B, J, nullptr, none, halo, err, far_list, src, perm);
     const int tile[3] = {tx, ty, tz};
     cudaError_t e = cudaSuccess;
     if (launch_persistent_fixed(dims, st, smem, nruns, run_cell_base, a, grid_blocks, launch, tile, halo, p0, p1,

@@ -12,7 +12,9 @@
 // cell, at once; up to 144 or 40 for one that changed cell, through its warp's
 // queue, drained 32 particles at a time.  A particle that has drifted
 // more than `halo` cells outside the tile since the last sort takes the same
-// arithmetic on the global arrays instead (periodic indices, global atomics).
+// arithmetic on the global arrays instead (periodic indices, global atomics);
+// an item that had such particles stages the tile where its particles are now
+// (item_shift).
 // At the end the block adds its current tile to the global J with atomics.
 #pragma once
 
@@ -26,7 +28,7 @@ namespace pic {
 
 template <typename R>
 struct PartArgs {
-    const WorkItem *items;
+    WorkItem *items;   // (`drifted` is written by the fused step)
     const int *n_items;
     const RunDev *runs;
     const GroupDev *groups;
@@ -38,11 +40,27 @@ struct PartArgs {
     Fields<R> F;
     int *old_cell;
     R *old_off[3];
+    unsigned *far_list;   // pool-sized scratch: particles past their item's staged tile (process_item)
     int halo;
     int *err;   // err[0]: error word; err[1]: particles that ran past their tile's halo (counted by MODES 0, 1)
 };
 
 extern __shared__ __align__(16) unsigned char g_smem[];
+
+// Blocks per SM the kernels are compiled for: two (128 registers), three of the
+// 2D FP32 ones (80).  Where the shared tiles leave room for one block only, the
+// launches take the variant compiled for one, whose registers hold everything:
+// 8x8x8 FP32 tiles and every 3D FP64 tile spilled 100 to 200 bytes per thread
+// at 128 registers (48^3 cells, 16 + 16 particles each, FP64: 5.3 -> 4.7 ms a
+// step).  The 2D FP32 persistent step of 24 runs took 22.5 ms per 30 steps at
+// two blocks, 19.7 at three and 21.0 at four.
+template <int DIM, typename R>
+constexpr int min_blocks()
+{
+    return DIM == 2 && sizeof(R) == 4 ? 3 : 2;
+}
+// The shared memory of an SM, and what the system keeps of it per block.
+inline bool one_block_per_sm(size_t smem) { return 2 * (smem + 1024) > 228 * 1024; }
 
 // Tile geometry of the particle kernels: extents T0 x T1 x T2, halo G and the
 // shared tiles' x and y pitches P0, P1.  GeoDyn reads them from the run and the
@@ -69,6 +87,16 @@ constexpr int kQueueVals = 7;
 __device__ __forceinline__ bool finite3(float a, float b, float c) { return isfinite(a) && isfinite(b) && isfinite(c); }
 __device__ __forceinline__ bool finite3(double a, double b, double c) { return isfinite(a) && isfinite(b) && isfinite(c); }
 
+// 4, 8 or 16 bytes from global to shared memory, both aligned to as much,
+// without waiting; complete after cp.async.wait_all of the thread.
+template <int BYTES>
+__device__ __forceinline__ void copy_async(void *dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+                 "n"(BYTES)
+                 : "memory");
+}
+
 // Tile-local coordinate of global index i for a tile starting at o with extent T:
 // the periodic image in [-G, T+G) if there is one (the grid is wider than the
 // staged region, so at most one image lies there), else a value outside it.
@@ -80,79 +108,199 @@ __device__ __forceinline__ int local_coord(int i, int o, int T, int G, int n)
     return l;
 }
 
-// Rare path: a particle more than `halo` cells outside its tile since the
-// last sort.  Same arithmetic on the periodic global arrays; kept out of line
-// so that it does not raise the register count of the tiled path.
-template <int DIM, typename R>
-__device__ __noinline__ void gather_global(const Fields<R> &F, long long cb, int i, int j, int k, int nx, int ny,
-                                           int nz, const R *w6, R *Ep, R *Bp)
+// Where the particles of a drifted item are now: the mean displacement of
+// (up to) kThreads of them, evenly spaced over the item, from the centre of its
+// tile, in whole cells.  The item then stages the tile moved by that much.  Any
+// shift gives the same step; it only decides which particles find their stencil
+// in shared memory.  A plasma that streams or is pushed by a laser carries a
+// tile's particles along together: for a slab behind a wave of a0 = 5, 4x4x4
+// tiles, halo 2 and a sort every 10 steps, the tenth step took 8.0 ms with the
+// tile staged where it was sorted (the first 0.8 ms).  One cell per thread is
+// read, and only by items that had an eighth of their particles (summed over the
+// steps since the sort) on the global-memory path: for the few that leave a tile
+// of a thermal plasma, which has no common drift to follow, the read cost more
+// than it gave (8x8x8 tiles, 20 steps: 8.07 -> 8.9 ms when one was enough).
+template <int DIM, typename R, bool OLD>
+__device__ __forceinline__ void item_shift(const PartArgs<R> &a, const WorkItem &it, const RunDev &rn, const int T[3],
+                                           int o[3])
 {
-    GlobalReader<R> rd;
-    for (int c = 0; c < 3; ++c) { rd.E[c] = F.E[c]; rd.B[c] = F.B[c]; }
-    for (int q = 0; q < 4; ++q) {
-        rd.xi[q] = cb + wrapi(i - 1 + q, nx);
-        rd.yj[q] = (long long)nx * wrapi(j - 1 + q, ny);
-        rd.zk[q] = DIM == 3 ? (long long)nx * ny * wrapi(k - 1 + q, nz) : 0;
+    __shared__ int sum[4];
+    if (threadIdx.x < 4) sum[threadIdx.x] = 0;
+    __syncthreads();
+    const long long len = it.end - it.begin;
+    int d[4] = {0, 0, 0, 0};
+    if (threadIdx.x < len) {
+        const long long p = it.begin + (len <= kThreads ? threadIdx.x : len * threadIdx.x / kThreads);
+        const int cell = OLD ? a.old_cell[p] : a.P.cell[p];
+        const int rest = divu31(cell, rn.div_nx);
+        const int k = DIM == 3 ? divu31(rest, rn.div_ny) : 0;
+        const int c[3] = {cell - rest * rn.n[0], rest - k * rn.n[1], k};
+#pragma unroll
+        for (int x = 0; x < DIM; ++x) {
+            d[x] = 2 * (c[x] - o[x]) - (T[x] - 1);   // twice the distance from the tile's centre, nearest image
+            if (d[x] > rn.n[x]) d[x] -= 2 * rn.n[x];
+            if (d[x] < -rn.n[x]) d[x] += 2 * rn.n[x];
+        }
+        d[3] = 1;
     }
-    R fx[2] = {w6[0], w6[1]}, fy[2] = {w6[5], w6[6]}, fz[2] = {w6[10], w6[11]};
-    R Sx[3] = {w6[2], w6[3], w6[4]}, Sy[3] = {w6[7], w6[8], w6[9]}, Sz[3] = {w6[12], w6[13], w6[14]};
-    gather<DIM>(rd, fx, Sx, fy, Sy, fz, Sz, Ep, Bp);
-}
-
-// full: bit a set when the particle changed cell along axis a (its window
-// there has four cells and three faces; along the other axes the fourth cell
-// and the third face carry nothing and are skipped, as on the tiled path)
-template <int DIM, typename R>
-__device__ __noinline__ void deposit_global(const Fields<R> &F, long long cb, int i, int j, int k, int nx, int ny,
-                                            int nz, const AxisWin<R> *win, const R *kf, R uz, int full)
-{
-    const AxisWin<R> X = win[0], Y = win[1], Z = win[2];
-    GlobalAcc<R, 4> acc;
-    for (int c = 0; c < 3; ++c) acc.J[c] = F.J[c];
-    acc.set(cb, i, j, k, nx, ny, nz, X.lo, Y.lo, Z.lo, DIM == 3);
-    deposit<DIM>(acc, X, Y, Z, kf, uz, full);
-}
-
-// The same for l_a = 2 1/2; (i, j, k) is the particle's base index.
-template <int DIM, typename R>
-__device__ __noinline__ void gather_global5(const Fields<R> &F, long long cb, int i, int j, int k, int nx, int ny,
-                                            int nz, const R *w, R *Ep, R *Bp)
-{
-    GlobalReader5<R> rd;
-    for (int c = 0; c < 3; ++c) { rd.E[c] = F.E[c]; rd.B[c] = F.B[c]; }
-    for (int q = 0; q < 5; ++q) {
-        rd.xi[q] = cb + wrapi(i - 2 + q, nx);
-        rd.yj[q] = (long long)nx * wrapi(j - 2 + q, ny);
-        rd.zk[q] = DIM == 3 ? (long long)nx * ny * wrapi(k - 2 + q, nz) : 0;
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+        const int v = __reduce_add_sync(0xffffffffu, d[x]);
+        if ((threadIdx.x & 31) == 0) atomicAdd(&sum[x], v);
     }
-    // w: f (3) and S (4) per axis
-    gather5<DIM>(rd, w, w + 3, w + 7, w + 10, w + 14, w + 17, Ep, Bp);
+    __syncthreads();
+    const float w = 0.5f / (float)max(sum[3], 1);
+#pragma unroll
+    for (int x = 0; x < DIM; ++x) o[x] = wrapi(o[x] + (int)rintf((float)sum[x] * w), rn.n[x]);
+    __syncthreads();
 }
 
-template <int DIM, typename R>
-__device__ __noinline__ void deposit_global5(const Fields<R> &F, long long cb, int i, int j, int k, int nx, int ny,
-                                             int nz, const AxisWin5<R> *win, const R *kf, R uz, int full)
+// A particle past the staged tile: the same arithmetic on the periodic global
+// arrays, for particle p of the item's group, read from a.S at sp with RP.  Out of
+// line, so that it does not raise the register count of the tiled path, and
+// called for all of an item's such particles together (see process_item).  On the global
+// arrays the fourth cell and third face along an axis that the particle did
+// not cross carry nothing and are skipped, as on the tiled path (`full`).
+template <int DIM, typename R, int MODE, int ORD, bool RP>
+__device__ __noinline__ void far_particle(const PartArgs<R> &a, int group, long long p, long long sp)
 {
-    const AxisWin5<R> X = win[0], Y = win[1], Z = win[2];
-    GlobalAcc<R, 5> acc;
-    for (int c = 0; c < 3; ++c) acc.J[c] = F.J[c];
-    acc.set(cb, i, j, k, nx, ny, nz, X.lo, Y.lo, Z.lo, DIM == 3);
-    deposit5<DIM>(acc, X, Y, Z, kf, uz, full);
-}
-
-// The comparison scheme of Eq. wrong1 on the global arrays; (i, j, k) is the cell.
-template <int DIM, typename R>
-__device__ __noinline__ void gather_global_w1(const Fields<R> &F, long long cb, int i, int j, int k, int nx, int ny,
-                                              int nz, const R *S, R *Ep, R *Bp)
-{
-    GlobalReader5<R> rd;
-    for (int c = 0; c < 3; ++c) { rd.E[c] = F.E[c]; rd.B[c] = F.B[c]; }
-    for (int q = 0; q < 5; ++q) {
-        rd.xi[q] = cb + wrapi(i - 2 + q, nx);
-        rd.yj[q] = (long long)nx * wrapi(j - 2 + q, ny);
-        rd.zk[q] = DIM == 3 ? (long long)nx * ny * wrapi(k - 2 + q, nz) : 0;
+    constexpr bool F32 = sizeof(R) == 4;
+    const GroupDev &gr = a.groups[group];
+    const RunDev &rn = a.runs[gr.run];
+    const int nx = rn.n[0], ny = rn.n[1], nz = rn.n[2];
+    const long long cb = rn.cell_base;
+    R c2, cl, hq;
+    if constexpr (F32) { cl = rn.cf; hq = gr.hqf; } else { cl = rn.c; hq = gr.hq; }
+    c2 = cl * cl;
+    const Pool<R> &src = RP ? a.S : a.P;
+    const int cell0 = MODE == 2 ? a.old_cell[p] : src.cell[sp];
+    const R o0 = MODE == 2 ? a.old_off[0][p] : src.off[0][sp];
+    const R o1 = MODE == 2 ? a.old_off[1][p] : src.off[1][sp];
+    const R o2 = DIM == 3 ? (MODE == 2 ? a.old_off[2][p] : src.off[2][sp]) : R(0);
+    R w[3] = {R(0), R(0), R(0)};
+    if (MODE != 2 || DIM == 2) {
+        w[0] = src.w[0][sp];
+        w[1] = src.w[1][sp];
+        w[2] = src.w[2][sp];
     }
-    gather_w1<DIM>(rd, S, S + 3, S + 6, Ep, Bp);
+    const int rest = divu31(cell0, rn.div_nx);
+    const int i = cell0 - rest * nx;
+    const int k = DIM == 3 ? divu31(rest, rn.div_ny) : 0, j = DIM == 3 ? rest - k * ny : rest;
+    // l_a = 2 1/2: the base index is the cell or the next one
+    R a0 = o0, a1 = o1, a2 = o2;
+    int u0 = 0, u1 = 0, u2 = 0;
+    if constexpr (ORD == 5) {
+        a2 = R(0.5);
+        u0 = split5(o0, a0);
+        u1 = split5(o1, a1);
+        if (DIM == 3) u2 = split5(o2, a2);
+    }
+    int s0 = 0, s1 = 0, s2 = 0;
+    R n0 = o0, n1 = o1, n2 = o2, uz = R(0);
+    if (MODE != 2) {
+        R Ep[3], Bp[3];
+        if constexpr (ORD == 3) {
+            GlobalReader<R> rd;
+            for (int c = 0; c < 3; ++c) { rd.E[c] = a.F.E[c]; rd.B[c] = a.F.B[c]; }
+            for (int q = 0; q < 4; ++q) {
+                rd.xi[q] = cb + wrapi(i - 1 + q, nx);
+                rd.yj[q] = (long long)nx * wrapi(j - 1 + q, ny);
+                rd.zk[q] = DIM == 3 ? (long long)nx * ny * wrapi(k - 1 + q, nz) : 0;
+            }
+            R fx[2], Sx[3], fy[2], Sy[3], fz[2] = {R(1), R(0)}, Sz[3] = {R(0), R(1), R(0)};
+            form_factor(o0, fx, Sx);
+            form_factor(o1, fy, Sy);
+            if (DIM == 3) form_factor(o2, fz, Sz);
+            gather<DIM>(rd, fx, Sx, fy, Sy, fz, Sz, Ep, Bp);
+        } else {
+            GlobalReader5<R> rd;   // offsets -2..2 from the base index (l_a = 2 1/2) or the cell (Eq. wrong1)
+            for (int c = 0; c < 3; ++c) { rd.E[c] = a.F.E[c]; rd.B[c] = a.F.B[c]; }
+            for (int q = 0; q < 5; ++q) {
+                rd.xi[q] = cb + wrapi(i + u0 - 2 + q, nx);
+                rd.yj[q] = (long long)nx * wrapi(j + u1 - 2 + q, ny);
+                rd.zk[q] = DIM == 3 ? (long long)nx * ny * wrapi(k + u2 - 2 + q, nz) : 0;
+            }
+            if constexpr (ORD == 5) {
+                R f[21];   // f (3) and S (4) along x, y, z
+                form_factor5(a0, f, f + 3);
+                form_factor5(a1, f + 7, f + 10);
+                form_factor5(a2, f + 14, f + 17);
+                gather5<DIM>(rd, f, f + 3, f + 7, f + 10, f + 14, f + 17, Ep, Bp);
+            } else {
+                R f[2], S[9] = {R(0), R(1), R(0), R(0), R(1), R(0), R(0), R(1), R(0)};
+                form_factor(o0, f, S);
+                form_factor(o1, f, S + 3);
+                if (DIM == 3) form_factor(o2, f, S + 6);
+                gather_w1<DIM>(rd, S, S + 3, S + 6, Ep, Bp);
+            }
+        }
+        boris(w, Ep, Bp, hq, c2);
+        const bool live = finite3(w[0], w[1], w[2]);
+        int cell1 = cell0;
+        if (live) {
+            R cN0, cN1, cN2;
+            if constexpr (F32) { cN0 = rn.cNf[0]; cN1 = rn.cNf[1]; cN2 = rn.cNf[2]; }
+            else { cN0 = rn.cN[0]; cN1 = rn.cN[1]; cN2 = rn.cN[2]; }
+            const R ig = rsqrt_r(w[0] * w[0] + w[1] * w[1] + w[2] * w[2] + c2);
+            s0 = renormalize(o0, w[0] * ig * cN0, n0);
+            s1 = renormalize(o1, w[1] * ig * cN1, n1);
+            if (DIM == 3) s2 = renormalize(o2, w[2] * ig * cN2, n2);
+            uz = cl * w[2] * ig;
+            cell1 = wrapi(i + s0, nx) + nx * (wrapi(j + s1, ny) + ny * (DIM == 3 ? wrapi(k + s2, nz) : 0));
+            if (MODE == 1) {
+                a.old_cell[p] = cell0;
+                a.old_off[0][p] = o0;
+                a.old_off[1][p] = o1;
+                if (DIM == 3) a.old_off[2][p] = o2;
+            }
+        } else {
+            atomicOr(a.err, ERR_NONFINITE);   // as in process_item: it keeps x^n and contributes no current
+        }
+        if (live || RP) {
+            if (RP) a.P.id[p] = a.S.id[sp];
+            a.P.cell[p] = cell1;
+            a.P.off[0][p] = n0;
+            a.P.off[1][p] = n1;
+            if (DIM == 3) a.P.off[2][p] = n2;
+            for (int c = 0; c < 3; ++c) a.P.w[c][p] = w[c];
+        }
+        if (MODE == 1 || !live) return;
+    } else {
+        const int cell1 = a.P.cell[p];
+        n0 = a.P.off[0][p];
+        n1 = a.P.off[1][p];
+        if (DIM == 3) n2 = a.P.off[2][p];
+        const int r1 = divu31(cell1, rn.div_nx);
+        const int k1 = DIM == 3 ? divu31(r1, rn.div_ny) : 0;
+        s0 = cell1 - r1 * nx - i; if (s0 > 1) s0 -= nx; if (s0 < -1) s0 += nx;
+        s1 = r1 - k1 * ny - j; if (s1 > 1) s1 -= ny; if (s1 < -1) s1 += ny;
+        if (DIM == 3) { s2 = k1 - k; if (s2 > 1) s2 -= nz; if (s2 < -1) s2 += nz; }
+        if (DIM == 2) uz = cl * w[2] * rsqrt_r(w[0] * w[0] + w[1] * w[1] + w[2] * w[2] + c2);
+    }
+    R kf[3];
+    for (int c = 0; c < 3; ++c) { if constexpr (F32) kf[c] = gr.kff[c]; else kf[c] = gr.kf[c]; }
+    if constexpr (ORD == 5) {
+        R b0, b1, b2 = R(0.5);
+        const int q0 = s0 + split5(n0, b0) - u0, q1 = s1 + split5(n1, b1) - u1;
+        const int q2 = DIM == 3 ? s2 + split5(n2, b2) - u2 : 0;
+        AxisWin5<R> X, Y, Z;
+        axis_window5(a0, b0, q0, X);
+        axis_window5(a1, b1, q1, Y);
+        if (DIM == 3) axis_window5(a2, b2, q2, Z); else Z = X;
+        GlobalAcc<R, 5> acc;
+        for (int c = 0; c < 3; ++c) acc.J[c] = a.F.J[c];
+        acc.set(cb, i + u0, j + u1, k + u2, nx, ny, nz, X.lo, Y.lo, Z.lo, DIM == 3);
+        deposit5<DIM>(acc, X, Y, Z, kf, uz, (q0 != 0 ? 1 : 0) | (q1 != 0 ? 2 : 0) | (q2 != 0 ? 4 : 0));
+    } else {
+        AxisWin<R> X, Y, Z;
+        axis_window(o0, n0, s0, X);
+        axis_window(o1, n1, s1, Y);
+        if (DIM == 3) axis_window(o2, n2, s2, Z); else Z = X;
+        GlobalAcc<R, 4> acc;
+        for (int c = 0; c < 3; ++c) acc.J[c] = a.F.J[c];
+        acc.set(cb, i, j, k, nx, ny, nz, X.lo, Y.lo, Z.lo, DIM == 3);
+        deposit<DIM>(acc, X, Y, Z, kf, uz, (s0 != 0 ? 1 : 0) | (s1 != 0 ? 2 : 0) | (s2 != 0 ? 4 : 0));
+    }
 }
 
 // MODE 0: fused gather + push + move + deposit (pic_step).
@@ -185,7 +333,12 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
     const int tx = it.tile % rn.ntile[0];
     const int ty = (it.tile / rn.ntile[0]) % rn.ntile[1];
     const int tz = DIM == 3 ? it.tile / (rn.ntile[0] * rn.ntile[1]) : 0;
-    const int ox = tx * T0, oy = ty * T1, oz = tz * T2;
+    int org[3] = {tx * T0, ty * T1, tz * T2};
+    if (!RP && 8LL * it.drifted > it.end - it.begin) {   // uniform over the block; none right after a sort
+        const int T[3] = {T0, T1, T2};
+        item_shift<DIM, R, MODE == 2>(a, it, rn, T, org);
+    }
+    const int ox = org[0], oy = org[1], oz = org[2];
     constexpr int FH = ORD == 3 ? 1 : 2, JH = ORD == 5 ? 3 : 2;   // field and current halo beyond G
     const int fe0 = T0 + 2 * (G + FH), fe1 = T1 + 2 * (G + FH), fe2 = DIM == 3 ? T2 + 2 * (G + FH) : 1;
     const int je0 = T0 + 2 * (G + JH), je1 = T1 + 2 * (G + JH), je2 = DIM == 3 ? T2 + 2 * (G + JH) : 1;
@@ -227,6 +380,14 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
         }
     }
 
+    // Particles past the staged tile: their indices in the item go to the item's
+    // part of far_list, and far_particle steps them together after the others.  A
+    // warp with one such lane would otherwise run the global-memory path for it
+    // alone (the tenth step of item_shift's slab: 8.0 ms), and a call from inside
+    // the loop would spill what the loop keeps in registers.
+    __shared__ int nfar;
+    if (threadIdx.x == 0) nfar = 0;
+
     if (NEED_F) {
         for (int l = threadIdx.x; l < nf; l += blockDim.x) {
             const int lx = l % P0, r = l / P0, ly = r % P1, lz = r / P1;
@@ -244,7 +405,8 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
     }
     if (NEED_J) {
         int *z = sJh[0];   // 24 * nj bytes = 6 * nj words in both precisions, + nj counts in FP32
-        for (int l = threadIdx.x; l < (FIX ? 7 : 6) * nj; l += blockDim.x) z[l] = 0;
+        const int nw = (FIX ? 7 : 6) * nj;
+        for (int l = threadIdx.x; l < nw; l += blockDim.x) z[l] = 0;
     }
     __syncthreads();
 
@@ -274,11 +436,11 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
     // of moved particles.  The integer current sums do not depend on the order.
     // The warps' queues lie one after another (values, then codes), followed by
     // one count per warp for the merged drain at the end of the item.
+    const int warp = threadIdx.x >> 5;
     R *qv0 = nullptr, *qv = nullptr;
     int *qs0 = nullptr, *qs = nullptr, *qcnt = nullptr;
     if (NEED_J) {
         unsigned char *qb = g_smem + (NEED_F ? 6 * (size_t)nf * sizeof(R) : 0) + (FIX ? 28 : 24) * (size_t)nj;
-        const int warp = threadIdx.x >> 5;
         qv0 = reinterpret_cast<R *>(qb);
         qs0 = reinterpret_cast<int *>(qb + (size_t)(kThreads / 32) * kQueueCap * kQueueVals * sizeof(R));
         qcnt = qs0 + (kThreads / 32) * kQueueCap;
@@ -376,7 +538,7 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
             if (p + blockDim.x < it.end) sp_next = a.perm[p + blockDim.x];
         }
         bool live = false;   // the particle moves and deposits this step
-        bool inr = false;
+        bool far = false;    // it lies past the staged tile: far_particle steps it later
         int i = 0, j = 0, k = 0, li = 0, lj = 0, lk = 0;
         R o0 = R(0), o1 = R(0), o2 = R(0), n0 = R(0), n1 = R(0), n2 = R(0), uz = R(0);
         int s0 = 0, s1 = 0, s2 = 0;
@@ -406,11 +568,15 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
             li = local_coord(i, ox, T0, G, nx);
             lj = local_coord(j, oy, T1, G, ny);
             lk = DIM == 3 ? local_coord(k, oz, T2, G, nz) : 0;
-            inr = li >= -G && li < T0 + G && lj >= -G && lj < T1 + G && (DIM == 2 || (lk >= -G && lk < T2 + G));
+            const bool inr =
+                li >= -G && li < T0 + G && lj >= -G && lj < T1 + G && (DIM == 2 || (lk >= -G && lk < T2 + G));
+            far = !inr;
 
             n0 = o0; n1 = o1; n2 = o2;
-            live = true;
-            if (MODE != 2) {
+            live = inr;
+            if (far) {
+                // stepped later, with 31 others
+            } else if (MODE != 2) {
                 R Ep[3], Bp[3];
                 if constexpr (ORD == 5) {
                     R e0, e1, e2 = R(0.5);
@@ -419,32 +585,24 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
                     form_factor5(e0, w, w + 3);
                     form_factor5(e1, w + 7, w + 10);
                     form_factor5(e2, w + 14, w + 17);
-                    if (inr) {
-                        SmemReader<R> rd;
-                        for (int c = 0; c < 3; ++c) { rd.E[c] = sE[c]; rd.B[c] = sB[c]; }
-                        rd.base = (li + u0 + G + FH) +
-                                  P0 * ((lj + u1 + G + FH) + (DIM == 3 ? P1 * (lk + u2 + G + FH) : 0));
-                        rd.s1 = P0;
-                        rd.s2 = P0 * P1;
-                        gather5<DIM>(rd, w, w + 3, w + 7, w + 10, w + 14, w + 17, Ep, Bp);
-                    } else {
-                        gather_global5<DIM, R>(a.F, cb, i + u0, j + u1, k + u2, nx, ny, nz, w, Ep, Bp);
-                    }
+                    SmemReader<R> rd;
+                    for (int c = 0; c < 3; ++c) { rd.E[c] = sE[c]; rd.B[c] = sB[c]; }
+                    rd.base = (li + u0 + G + FH) +
+                              P0 * ((lj + u1 + G + FH) + (DIM == 3 ? P1 * (lk + u2 + G + FH) : 0));
+                    rd.s1 = P0;
+                    rd.s2 = P0 * P1;
+                    gather5<DIM>(rd, w, w + 3, w + 7, w + 10, w + 14, w + 17, Ep, Bp);
                 } else if constexpr (ORD == 4) {
                     R f[2], S[9] = {R(0), R(1), R(0), R(0), R(1), R(0), R(0), R(1), R(0)};   // S along x, y, z
                     form_factor(o0, f, S);
                     form_factor(o1, f, S + 3);
                     if (DIM == 3) form_factor(o2, f, S + 6);
-                    if (inr) {
-                        SmemReader<R> rd;
-                        for (int c = 0; c < 3; ++c) { rd.E[c] = sE[c]; rd.B[c] = sB[c]; }
-                        rd.base = (li + G + FH) + P0 * ((lj + G + FH) + (DIM == 3 ? P1 * (lk + G + FH) : 0));
-                        rd.s1 = P0;
-                        rd.s2 = P0 * P1;
-                        gather_w1<DIM>(rd, S, S + 3, S + 6, Ep, Bp);
-                    } else {
-                        gather_global_w1<DIM, R>(a.F, cb, i, j, k, nx, ny, nz, S, Ep, Bp);
-                    }
+                    SmemReader<R> rd;
+                    for (int c = 0; c < 3; ++c) { rd.E[c] = sE[c]; rd.B[c] = sB[c]; }
+                    rd.base = (li + G + FH) + P0 * ((lj + G + FH) + (DIM == 3 ? P1 * (lk + G + FH) : 0));
+                    rd.s1 = P0;
+                    rd.s2 = P0 * P1;
+                    gather_w1<DIM>(rd, S, S + 3, S + 6, Ep, Bp);
                 } else {
                     R fx[2], Sx[3], fy[2], Sy[3], fz[2], Sz[3];
                     form_factor(o0, fx, Sx);
@@ -455,18 +613,12 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
                         fz[0] = R(1); fz[1] = R(0);
                         Sz[0] = R(0); Sz[1] = R(1); Sz[2] = R(0);
                     }
-                    if (inr) {
-                        SmemReader<R> rd;
-                        for (int c = 0; c < 3; ++c) { rd.E[c] = sE[c]; rd.B[c] = sB[c]; }
-                        rd.base = (li + G + 1) + P0 * ((lj + G + 1) + (DIM == 3 ? P1 * (lk + G + 1) : 0));
-                        rd.s1 = P0;
-                        rd.s2 = P0 * P1;
-                        gather<DIM>(rd, fx, Sx, fy, Sy, fz, Sz, Ep, Bp);
-                    } else {
-                        R w6[15] = {fx[0], fx[1], Sx[0], Sx[1], Sx[2], fy[0], fy[1], Sy[0], Sy[1], Sy[2],
-                                    fz[0], fz[1], Sz[0], Sz[1], Sz[2]};
-                        gather_global<DIM, R>(a.F, cb, i, j, k, nx, ny, nz, w6, Ep, Bp);
-                    }
+                    SmemReader<R> rd;
+                    for (int c = 0; c < 3; ++c) { rd.E[c] = sE[c]; rd.B[c] = sB[c]; }
+                    rd.base = (li + G + 1) + P0 * ((lj + G + 1) + (DIM == 3 ? P1 * (lk + G + 1) : 0));
+                    rd.s1 = P0;
+                    rd.s2 = P0 * P1;
+                    gather<DIM>(rd, fx, Sx, fy, Sy, fz, Sz, Ep, Bp);
                 }
                 boris(w, Ep, Bp, hq, c2);
                 if (!finite3(w[0], w[1], w[2])) {
@@ -522,9 +674,12 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
                 }
             }
         }
-        if (MODE != 2) {   // particles on the global path: the sort policy's measure of drift
-            const unsigned dm = __ballot_sync(0xffffffffu, valid && !inr);
-            if (lane == 0 && dm != 0u) atomicAdd(reinterpret_cast<unsigned *>(a.err) + 1, (unsigned)__popc(dm));
+        const unsigned fm = __ballot_sync(0xffffffffu, far);
+        if (fm != 0u) {   // warp-uniform
+            int at = 0;
+            if (lane == 0) at = atomicAdd(&nfar, __popc(fm));
+            at = __shfl_sync(0xffffffffu, at, 0) + __popc(fm & ((1u << lane) - 1u));
+            if (far) a.far_list[it.begin + at] = (unsigned)(p - it.begin);
         }
         if (MODE == 1) continue;
 
@@ -550,7 +705,7 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
         const bool moved = (q0 | q1 | q2) != 0;
         const int base = (li + ub0 + G + JH) +
                          P0 * ((lj + ub1 + G + JH) + (DIM == 3 ? P1 * (lk + ub2 + G + JH) : 0));
-        if (live && inr && !moved) {
+        if (live && !moved) {
             if constexpr (ORD == 5) {
                 AxisWin5<R> X, Y, Z;
                 axis_window5(a0, b0, 0, X);
@@ -586,24 +741,8 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
                     deposit_local(base, X, Y, Z, uz, 0);
                 }
             }
-        } else if (live && !inr) {
-            if constexpr (ORD == 5) {
-                AxisWin5<R> win[3];
-                axis_window5(a0, b0, q0, win[0]);
-                axis_window5(a1, b1, q1, win[1]);
-                if (DIM == 3) axis_window5(a2, b2, q2, win[2]); else win[2] = win[0];
-                deposit_global5<DIM, R>(a.F, cb, i + ub0, j + ub1, k + ub2, nx, ny, nz, win, kf, uz,
-                                        (q0 != 0 ? 1 : 0) | (q1 != 0 ? 2 : 0) | (q2 != 0 ? 4 : 0));
-            } else {
-                AxisWin<R> win[3];
-                axis_window(o0, n0, s0, win[0]);
-                axis_window(o1, n1, s1, win[1]);
-                if (DIM == 3) axis_window(o2, n2, s2, win[2]); else win[2] = win[0];
-                deposit_global<DIM, R>(a.F, cb, i, j, k, nx, ny, nz, win, kf, uz,
-                                       (s0 != 0 ? 1 : 0) | (s1 != 0 ? 2 : 0) | (s2 != 0 ? 4 : 0));
-            }
         }
-        const bool enq = live && inr && moved;
+        const bool enq = live && moved;
         const unsigned qm = __ballot_sync(0xffffffffu, enq);
         if (enq) {
             const int slot = qn + __popc(qm & ((1u << lane) - 1u));
@@ -627,14 +766,24 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
             __syncwarp();   // the drained slots are free again
         }
     }
+    if (NEED_J && lane == 0) qcnt[warp] = qn;
+    __syncthreads();
+    if (nfar > 0) {
+        for (int m = threadIdx.x; m < nfar; m += blockDim.x) {
+            const long long pf = it.begin + a.far_list[it.begin + m];
+            far_particle<DIM, R, MODE, ORD, RP>(a, it.group, pf, RP ? (long long)a.perm[pf] : pf);
+        }
+        if (MODE != 2 && threadIdx.x == 0) {   // the sort policy's measure of drift, and item_shift's
+            atomicAdd(reinterpret_cast<unsigned *>(a.err) + 1, (unsigned)nfar);
+            a.items[item].drifted = it.drifted + nfar;
+        }
+    }
     if (NEED_J) {
         // The entries left in the warps' queues (fewer than 32 each) are drained
         // together: merged entry m is slot m - (entries of the warps before) of
         // its warp's queue, and warp w deposits the merged entries
         // [32w, 32w + 32), [32w + 256, ...).  A block then runs about one
         // partly filled drain per item instead of one per warp.
-        if (lane == 0) qcnt[threadIdx.x >> 5] = qn;
-        __syncthreads();
         int tot = 0;
 #pragma unroll
         for (int w = 0; w < kThreads / 32; ++w) tot += qcnt[w];
@@ -755,8 +904,8 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
     __syncthreads();   // the shared tiles are free for the block's next item
 }
 
-template <int DIM, typename R, int MODE, class GEO = GeoDyn, int ORD = 3, bool PERM = false>
-__global__ void __launch_bounds__(kThreads) k_particles(const PartArgs<R> a)
+template <int DIM, typename R, int MODE, class GEO = GeoDyn, int ORD = 3, bool PERM = false, bool ONE = false>
+__global__ void __launch_bounds__(kThreads, ONE ? 1 : min_blocks<DIM, R>()) k_particles(const __grid_constant__ PartArgs<R> a)
 {
     if ((int)blockIdx.x >= *a.n_items) return;
     process_item<DIM, R, MODE, GEO, ORD, PERM>(a, blockIdx.x);
@@ -779,8 +928,8 @@ __device__ __forceinline__ int find_run(const long long *run_cell_base, int nrun
 // that all blocks are resident (cooperative launch), which the barriers need.
 // PERM: the step right after a sort that left the arrays in place; the work
 // items read the particles through the permutation (as k_particles does).
-template <int DIM, typename R, class GEO = GeoDyn, bool PERM = false>
-__global__ void __launch_bounds__(kThreads) k_step_persistent(const PartArgs<R> a, int nruns,
+template <int DIM, typename R, class GEO = GeoDyn, bool PERM = false, bool ONE = false>
+__global__ void __launch_bounds__(kThreads, ONE ? 1 : min_blocks<DIM, R>()) k_step_persistent(const __grid_constant__ PartArgs<R> a, int nruns,
                                                               const long long *run_cell_base, long long *ant_n,
                                                               int antennas)
 {
@@ -816,32 +965,57 @@ template <int DIM, typename R, int MODE, class GEO = GeoDyn, int ORD = 3>
 static cudaError_t launch_t(cudaStream_t st, int max_items, size_t smem, const PartArgs<R> &a)
 {
     if (max_items <= 0) return cudaSuccess;
+    constexpr bool both = GEO::dyn && DIM == 3;
     if constexpr (MODE == 0 && ORD == 3) {
         if (a.perm) {   // right after a sort: the kernel that reads through the permutation
-            k_particles<DIM, R, 0, GEO, 3, true><<<max_items, kThreads, smem, st>>>(a);
+            if (both && one_block_per_sm(smem))
+                k_particles<DIM, R, 0, GEO, 3, true, both><<<max_items, kThreads, smem, st>>>(a);
+            else
+                k_particles<DIM, R, 0, GEO, 3, true><<<max_items, kThreads, smem, st>>>(a);
             return cudaGetLastError();
         }
     }
-    k_particles<DIM, R, MODE, GEO, ORD><<<max_items, kThreads, smem, st>>>(a);
+    if (both && one_block_per_sm(smem))
+        k_particles<DIM, R, MODE, GEO, ORD, false, both><<<max_items, kThreads, smem, st>>>(a);
+    else
+        k_particles<DIM, R, MODE, GEO, ORD><<<max_items, kThreads, smem, st>>>(a);
     return cudaGetLastError();
+}
+
+// The shared-memory limit of a particle kernel, of each variant.
+template <int DIM, typename R, int MODE, class GEO, int ORD = 3, bool PERM = false>
+static cudaError_t set_limit_one(int bytes)
+{
+    cudaError_t e = cudaFuncSetAttribute(k_particles<DIM, R, MODE, GEO, ORD, PERM>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if constexpr (GEO::dyn && DIM == 3) {
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_particles<DIM, R, MODE, GEO, ORD, PERM, true>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    }
+    return e;
 }
 
 // The shared-memory limit of the fused kernel of a geometry, both variants.
 template <int DIM, typename R, class GEO>
 static cudaError_t set_limit_fused(int bytes)
 {
-    cudaError_t e = cudaFuncSetAttribute(k_particles<DIM, R, 0, GEO>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    cudaError_t e = set_limit_one<DIM, R, 0, GEO>(bytes);
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_particles<DIM, R, 0, GEO, 3, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                bytes);
+    return set_limit_one<DIM, R, 0, GEO, 3, true>(bytes);
 }
 
 template <int DIM, typename R, class GEO = GeoDyn>
 static cudaError_t persistent_t(cudaStream_t st, size_t smem, int nruns, const long long *run_cell_base,
                                 PartArgs<R> a, int *grid_blocks, int launch, long long *ant_n, int antennas)
 {
+    constexpr bool both = GEO::dyn && DIM == 3;
     auto fn0 = k_step_persistent<DIM, R, GEO, false>;
     auto fn1 = k_step_persistent<DIM, R, GEO, true>;
+    if (both && one_block_per_sm(smem)) {
+        fn0 = k_step_persistent<DIM, R, GEO, false, both>;
+        fn1 = k_step_persistent<DIM, R, GEO, true, both>;
+    }
     auto fn = a.perm ? fn1 : fn0;
     cudaError_t e;
     if (*grid_blocks <= 0) {
@@ -868,12 +1042,13 @@ static cudaError_t persistent_t(cudaStream_t st, size_t smem, int nruns, const l
 
 // Kernel arguments from the host-side buffers.
 template <typename R>
-inline PartArgs<R> make_args(const WorkItem *items, const int *n_items, const RunDev *runs, const GroupDev *groups,
+inline PartArgs<R> make_args(WorkItem *items, const int *n_items, const RunDev *runs, const GroupDev *groups,
                              const PoolBuf &P, void *const E[3], void *const B[3], void *const J[3], int *old_cell,
-                             void *const old_off[3], int halo, int *err, const PoolBuf *S = nullptr,
-                             const unsigned *perm = nullptr)
+                             void *const old_off[3], int halo, int *err, unsigned *far_list,
+                             const PoolBuf *S = nullptr, const unsigned *perm = nullptr)
 {
     PartArgs<R> a;
+    a.far_list = far_list;
     a.items = items;
     a.n_items = n_items;
     a.runs = runs;
@@ -925,17 +1100,19 @@ static cudaError_t launch_mode_ord(int mode, cudaStream_t st, int max_items, siz
 
 template <int ORD>
 static cudaError_t launch_particles_ord_t(int dims, int prec, int mode, cudaStream_t st, int max_items, size_t smem,
-                                          const WorkItem *items, const int *n_items, const RunDev *runs,
+                                          WorkItem *items, const int *n_items, const RunDev *runs,
                                           const GroupDev *groups, const PoolBuf &P, void *const E[3],
                                           void *const B[3], void *const J[3], int *old_cell, void *const old_off[3],
-                                          int halo, int *err)
+                                          int halo, int *err, unsigned *far_list)
 {
     if (prec == 0) {
-        auto a = make_args<double>(items, n_items, runs, groups, P, E, B, J, old_cell, old_off, halo, err);
+        auto a = make_args<double>(items, n_items, runs, groups, P, E, B, J, old_cell, old_off, halo, err,
+                                     far_list);
         return dims == 3 ? launch_mode_ord<3, double, ORD>(mode, st, max_items, smem, a)
                          : launch_mode_ord<2, double, ORD>(mode, st, max_items, smem, a);
     }
-    auto a = make_args<float>(items, n_items, runs, groups, P, E, B, J, old_cell, old_off, halo, err);
+    auto a = make_args<float>(items, n_items, runs, groups, P, E, B, J, old_cell, old_off, halo, err,
+                                     far_list);
     return dims == 3 ? launch_mode_ord<3, float, ORD>(mode, st, max_items, smem, a)
                      : launch_mode_ord<2, float, ORD>(mode, st, max_items, smem, a);
 }
@@ -945,9 +1122,9 @@ static cudaError_t set_limit_ord(int mode, size_t bytes)
 {
     const int b = (int)bytes;
     switch (mode) {
-    case 0: return cudaFuncSetAttribute(k_particles<DIM, R, 0, GeoDyn, ORD>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-    case 1: return cudaFuncSetAttribute(k_particles<DIM, R, 1, GeoDyn, ORD>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-    default: return cudaFuncSetAttribute(k_particles<DIM, R, 2, GeoDyn, ORD>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+    case 0: return set_limit_one<DIM, R, 0, GeoDyn, ORD>(b);
+    case 1: return set_limit_one<DIM, R, 1, GeoDyn, ORD>(b);
+    default: return set_limit_one<DIM, R, 2, GeoDyn, ORD>(b);
     }
 }
 
@@ -960,15 +1137,15 @@ static cudaError_t particles_ord_set_smem_limit_t(int dims, int prec, int mode, 
 }
 
 cudaError_t launch_particles_o5(int dims, int prec, int mode, cudaStream_t st, int max_items, size_t smem,
-                                const WorkItem *items, const int *n_items, const RunDev *runs, const GroupDev *groups,
+                                WorkItem *items, const int *n_items, const RunDev *runs, const GroupDev *groups,
                                 const PoolBuf &P, void *const E[3], void *const B[3], void *const J[3],
-                                int *old_cell, void *const old_off[3], int halo, int *err, const int tile[3], int p0,
-                                int p1);
+                                int *old_cell, void *const old_off[3], int halo, int *err, unsigned *far_list,
+                                const int tile[3], int p0, int p1);
 cudaError_t particles_o5_set_smem_limit(int dims, int prec, int mode, size_t bytes);
 cudaError_t launch_particles_w1(int dims, int prec, int mode, cudaStream_t st, int max_items, size_t smem,
-                                const WorkItem *items, const int *n_items, const RunDev *runs, const GroupDev *groups,
+                                WorkItem *items, const int *n_items, const RunDev *runs, const GroupDev *groups,
                                 const PoolBuf &P, void *const E[3], void *const B[3], void *const J[3],
-                                int *old_cell, void *const old_off[3], int halo, int *err);
+                                int *old_cell, void *const old_off[3], int halo, int *err, unsigned *far_list);
 cudaError_t particles_w1_set_smem_limit(int dims, int prec, int mode, size_t bytes);
 
 }  // namespace pic

@@ -34,6 +34,39 @@
 
 namespace pic {
 
+// Rare path: a particle more than `halo` cells outside its tile since the
+// last sort.  Same arithmetic on the periodic global arrays; kept out of line
+// so that it does not raise the register count of the tiled path.
+template <int DIM, typename R>
+__device__ __noinline__ void gather_global(const Fields<R> &F, long long cb, int i, int j, int k, int nx, int ny,
+                                           int nz, const R *w6, R *Ep, R *Bp)
+{
+    GlobalReader<R> rd;
+    for (int c = 0; c < 3; ++c) { rd.E[c] = F.E[c]; rd.B[c] = F.B[c]; }
+    for (int q = 0; q < 4; ++q) {
+        rd.xi[q] = cb + wrapi(i - 1 + q, nx);
+        rd.yj[q] = (long long)nx * wrapi(j - 1 + q, ny);
+        rd.zk[q] = DIM == 3 ? (long long)nx * ny * wrapi(k - 1 + q, nz) : 0;
+    }
+    R fx[2] = {w6[0], w6[1]}, fy[2] = {w6[5], w6[6]}, fz[2] = {w6[10], w6[11]};
+    R Sx[3] = {w6[2], w6[3], w6[4]}, Sy[3] = {w6[7], w6[8], w6[9]}, Sz[3] = {w6[12], w6[13], w6[14]};
+    gather<DIM>(rd, fx, Sx, fy, Sy, fz, Sz, Ep, Bp);
+}
+
+// full: bit a set when the particle changed cell along axis a (its window
+// there has four cells and three faces; along the other axes the fourth cell
+// and the third face carry nothing and are skipped, as on the tiled path)
+template <int DIM, typename R>
+__device__ __noinline__ void deposit_global(const Fields<R> &F, long long cb, int i, int j, int k, int nx, int ny,
+                                            int nz, const AxisWin<R> *win, const R *kf, R uz, int full)
+{
+    const AxisWin<R> X = win[0], Y = win[1], Z = win[2];
+    GlobalAcc<R, 4> acc;
+    for (int c = 0; c < 3; ++c) acc.J[c] = F.J[c];
+    acc.set(cb, i, j, k, nx, ny, nz, X.lo, Y.lo, Z.lo, DIM == 3);
+    deposit<DIM>(acc, X, Y, Z, kf, uz, full);
+}
+
 namespace {
 
 constexpr int kT0 = 8, kT1 = 4, kT2 = 4, kG = 1;

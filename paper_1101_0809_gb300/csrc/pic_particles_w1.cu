@@ -8,12 +8,12 @@
 namespace pic {
 
 cudaError_t launch_particles_w1(int dims, int prec, int mode, cudaStream_t st, int max_items, size_t smem,
-                                const WorkItem *items, const int *n_items, const RunDev *runs, const GroupDev *groups,
+                                WorkItem *items, const int *n_items, const RunDev *runs, const GroupDev *groups,
                                 const PoolBuf &P, void *const E[3], void *const B[3], void *const J[3],
-                                int *old_cell, void *const old_off[3], int halo, int *err)
+                                int *old_cell, void *const old_off[3], int halo, int *err, unsigned *far_list)
 {
     return launch_particles_ord_t<4>(dims, prec, mode, st, max_items, smem, items, n_items, runs, groups, P, E, B, J,
-                                      old_cell, old_off, halo, err);
+                                      old_cell, old_off, halo, err, far_list);
 }
 
 cudaError_t particles_w1_set_smem_limit(int dims, int prec, int mode, size_t bytes)

@@ -1100,6 +1100,7 @@ __global__ void k_items(const long long *tile_start, const unsigned *scan, int t
         w.tile = t - groups[lo].tile_base;
         w.begin = b + (long long)q * part;
         w.end = w.begin + part < e ? w.begin + part : e;
+        w.drifted = 0;
         items[s + q] = w;
     }
     if (t == total_tiles - 1) *n_items = (int)(s + cnt);
