@@ -174,26 +174,30 @@ void dfree(void *p)
 
 void free_pool(PoolBuf &P)
 {
-    dfree(P.cell);
-    dfree(P.id);
-    for (int c = 0; c < 3; ++c) {
-        dfree(P.off[c]);
-        dfree(P.w[c]);
-    }
+    dfree(P.slab);
     P = PoolBuf();
 }
 
 cudaError_t alloc_pool(pic_grid *g, PoolBuf &P, long long n)
 {
     P = PoolBuf();
-    cudaError_t e;
     n = (n + 3) & ~3LL;   // whole 16-byte groups: the re-sort copies segments rounded out to them
-    if ((e = dalloc(&P.cell, n)) != cudaSuccess) return e;
-    if ((e = dalloc(&P.id, n)) != cudaSuccess) return e;
-    for (int c = 0; c < 3; ++c) {
-        if (c < g->dims && (e = dalloc_bytes(&P.off[c], n * elem(g))) != cudaSuccess) return e;
-        if ((e = dalloc_bytes(&P.w[c], n * elem(g))) != cudaSuccess) return e;
-    }
+    if (n == 0) return cudaSuccess;
+    auto part = [](size_t bytes) { return (bytes + 255) & ~(size_t)255; };   // cudaMalloc's own alignment
+    const size_t wi = part(n * sizeof(int)), wr = part(n * elem(g));
+    const size_t bytes = std::max(2 * wi + (g->dims + 3) * wr, (size_t)n * sizeof(LoadRec));
+    const cudaError_t e = dalloc_bytes(&P.slab, bytes);
+    if (e != cudaSuccess) return e;
+    unsigned char *at = static_cast<unsigned char *>(P.slab);
+    auto take = [&](size_t w) {
+        unsigned char *p = at;
+        at += w;
+        return p;
+    };
+    P.cell = reinterpret_cast<int *>(take(wi));
+    P.id = reinterpret_cast<int *>(take(wi));
+    for (int c = 0; c < g->dims; ++c) P.off[c] = take(wr);
+    for (int c = 0; c < 3; ++c) P.w[c] = take(wr);
     return cudaSuccess;
 }
 
@@ -425,7 +429,9 @@ static int settle(pic_grid *g)
     return PIC_OK;
 }
 
-int do_sort(pic_grid *g, bool defer = false)
+// rec: the particles are the records in pool_alt's allocation (a load), their
+// cells in pool.cell; the sorted arrays go to pool.
+int do_sort(pic_grid *g, bool defer = false, bool rec = false)
 {
     int rc = settle(g);
     if (rc != PIC_OK) return rc;
@@ -437,7 +443,8 @@ int do_sort(pic_grid *g, bool defer = false)
     ProfScope ps(g, PIC_PROF_SORT);
     int nl = 0;
     const unsigned *perm = nullptr;
-    cudaError_t e = sort_and_build_items(g->prec, g->dims, g->stream, g->total, g->pool, g->pool_alt, g->d_groups,
+    cudaError_t e = sort_and_build_items(g->prec, g->dims, g->stream, g->total, g->pool,
+                                         rec ? g->pool : g->pool_alt, g->d_groups,
                                          g->d_group_base, (int)g->groups.size(), g->d_runs, g->total_tiles, g->sort,
                                          g->tile_start, g->item_scan, g->items, g->n_items, g->item_len,
                                          g->halo + (g->order2 == 5 ? 1 : 0),   // the current tile's bank base
@@ -445,13 +452,14 @@ int do_sort(pic_grid *g, bool defer = false)
                                          g->sort_order == PIC_SORT_CELL_LANES ? g->lane_cell : nullptr,
                                          g->sort_order == PIC_SORT_CELL_LANES ? g->lane_count : nullptr,
                                          g->tiles_valid && g->sort_order != PIC_SORT_CELL_LANES ? 1 : 0,
-                                         defer ? &perm : nullptr);
+                                         defer ? &perm : nullptr,
+                                         rec ? static_cast<const LoadRec *>(g->pool_alt.slab) : nullptr);
     launch_count_add(g, nl);
     g->tiles_valid = false;
     if (e != cudaSuccess) return cuda_fail(e, "tile sort");
     g->tiles_valid = true;
     if (perm) g->pending_perm = perm;   // the next fused particle launch moves the arrays
-    else if (g->total > 0 && !g->groups.empty()) std::swap(g->pool, g->pool_alt);
+    else if (!rec) std::swap(g->pool, g->pool_alt);
     if (!g->capturing) graph_drop(g);   // a captured graph assumes its own buffer parity
     g->steps_since_sort = 0;
     g->have_old = false;
@@ -1028,13 +1036,16 @@ static int load_many(pic_grid *g, std::vector<LoadReq> &reqs, int on_device)
         }
         so += 6 * q.n;
     }
-    auto convert = [&](size_t r, const PoolBuf &P, long long base) -> cudaError_t {
+    // FP32 loads go to the sort as records (LoadRec)
+    const bool rec = g->prec == PIC_FP32 && g->order2 != 5 && g->sort_order != PIC_SORT_CELL_LANES;
+    auto convert = [&](size_t r, const PoolBuf &P, const PoolBuf &alt, long long base) -> cudaError_t {
         const LoadReq &q = reqs[r];
         if (q.n == 0) return cudaSuccess;
         const RunDev &rn = g->runs[q.run].dev;
         launch_count_add(g, 1);
         return launch_load(g->prec, g->stream, q.n, src[r][0], src[r][1], src[r][2], src[r][3], src[r][4], src[r][5],
-                           g->dims, rn.n[0], rn.n[1], rn.n[2], P, base);
+                           g->dims, rn.n[0], rn.n[1], rn.n[2], P, base,
+                           rec ? static_cast<LoadRec *>(alt.slab) : nullptr);
     };
     // every request matches a loaded group of the same size: convert in place
     bool in_place = true;
@@ -1052,8 +1063,20 @@ static int load_many(pic_grid *g, std::vector<LoadReq> &reqs, int on_device)
         }
         int rc = upload_groups(g);
         if (rc != PIC_OK) return rc;
-        for (size_t r = 0; r < reqs.size(); ++r) CK(convert(r, g->pool, match[r]->base), "particle load");
-        rc = do_sort(g);
+        if (rec) {   // the groups that stay
+            for (auto &h : g->groups) {
+                bool stays = h.n > 0;
+                for (auto *m : match) stays = stays && m != &h;
+                if (!stays) continue;
+                CK(launch_copy_pool_rec(g->stream, g->pool, h.base, g->pool.cell,
+                                        static_cast<LoadRec *>(g->pool_alt.slab), h.base, h.n, g->dims),
+                   "particle load");
+                launch_count_add(g, 1);
+            }
+        }
+        for (size_t r = 0; r < reqs.size(); ++r)
+            CK(convert(r, g->pool, g->pool_alt, match[r]->base), "particle load");
+        rc = do_sort(g, false, rec);
         if (rc != PIC_OK) return rc;
         for (auto &q : reqs) g->have_ref[q.run] = 0;
         if (!on_device) CK(cudaStreamSynchronize(g->stream), "load");
@@ -1098,12 +1121,14 @@ static int load_many(pic_grid *g, std::vector<LoadReq> &reqs, int on_device)
         if (e != cudaSuccess) break;
         if (h.base >= 0) {   // an old group keeps its data
             if (h.n > 0) {
-                e = launch_copy_pool(g->prec, g->stream, g->pool, h.base, np, pb, h.n);
+                e = rec ? launch_copy_pool_rec(g->stream, g->pool, h.base, np.cell, static_cast<LoadRec *>(na.slab),
+                                               pb, h.n, g->dims)
+                        : launch_copy_pool(g->prec, g->stream, g->pool, h.base, np, pb, h.n);
                 launch_count_add(g, 1);
             }
         } else {
             for (size_t r = 0; r < reqs.size(); ++r)
-                if (reqs[r].run == h.run && reqs[r].species == h.species) e = convert(r, np, pb);
+                if (reqs[r].run == h.run && reqs[r].species == h.species) e = convert(r, np, na, pb);
         }
         h.base = pb;
         pb += h.n;
@@ -1130,7 +1155,7 @@ static int load_many(pic_grid *g, std::vector<LoadReq> &reqs, int on_device)
         set_last_error((msg + "; the grid's particles were dropped").c_str());
         return rc;
     }
-    rc = do_sort(g);
+    rc = do_sort(g, false, rec);
     if (rc != PIC_OK) return rc;
     for (auto &q : reqs) g->have_ref[q.run] = 0;
     CK(cudaStreamSynchronize(g->stream), "load: sort");

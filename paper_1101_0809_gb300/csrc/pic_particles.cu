@@ -121,25 +121,35 @@ cudaError_t launch_step_persistent(int dims, int prec, cudaStream_t st, WorkItem
 // precision, periodic wrap into [0, N); an offset that rounds to 1 moves to the
 // next cell with offset 0.  Momenta are converted; id = index in the call.
 // ---------------------------------------------------------------------------
-template <typename R>
+// With REC (FP32) the particle is written as one 32-byte record, for the sort's
+// gather.  A position already in [0, N) is taken as it is: the wrap would
+// subtract N * floor(x / N) = 0, and its FP64 quotient set the kernel's time
+// (16e6 particles: 1.66 ms with it; their 80 bytes each are 0.19 ms of memory).
+__device__ __forceinline__ double wrap_position(double x, double N)
+{
+    if (x >= 0.0 && x < N) return x;
+    x -= N * floor(x / N);
+    if (x >= N) x -= N;
+    if (x < 0.0) x = 0.0;
+    return x;
+}
+
+template <typename R, int DIM, bool REC>
 __global__ void k_load(long long n, const double *x0, const double *x1, const double *x2, const double *w0,
-                       const double *w1, const double *w2, int dims, int nx, int ny, int nz, int *cell,
-                       R *off0, R *off1, R *off2, R *wo0, R *wo1, R *wo2, int *id, long long base)
+                       const double *w1, const double *w2, int nx, int ny, int nz, PoolBuf P, LoadRec *rec,
+                       long long base)
 {
     const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (p >= n) return;
-    const double *xs[3] = {x0, x1, x2};
-    R *offs[3] = {off0, off1, off2};
+    const double xs[3] = {x0[p], x1[p], DIM == 3 ? x2[p] : 0.0};
+    const double ws[3] = {w0[p], w1[p], w2[p]};
     const int nn[3] = {nx, ny, nz};
     int ci[3] = {0, 0, 0};
-    for (int a = 0; a < dims; ++a) {
-        const double N = (double)nn[a];
-        double x = xs[a][p];
-        x -= N * floor(x / N);
-        if (x >= N) x -= N;
-        if (x < 0.0) x = 0.0;
-        double fl = floor(x);
-        int c = (int)fl;
+    R of[3] = {R(0), R(0), R(0)};
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) {
+        const double x = wrap_position(xs[a], (double)nn[a]);
+        int c = (int)floor(x);
         if (c >= nn[a]) c = nn[a] - 1;
         R o = (R)(x - (double)c);
         if (o >= R(1)) {
@@ -147,33 +157,74 @@ __global__ void k_load(long long n, const double *x0, const double *x1, const do
             c = c + 1 == nn[a] ? 0 : c + 1;
         }
         ci[a] = c;
-        offs[a][base + p] = o;
+        of[a] = o;
     }
-    cell[base + p] = ci[0] + nx * (ci[1] + ny * ci[2]);
-    wo0[base + p] = (R)w0[p];
-    wo1[base + p] = (R)w1[p];
-    wo2[base + p] = (R)w2[p];
-    id[base + p] = (int)p;
+    const int cell = ci[0] + nx * (ci[1] + ny * ci[2]);
+    P.cell[base + p] = cell;
+    if constexpr (REC) {
+        int4 *r = reinterpret_cast<int4 *>(rec + base + p);
+        r[0] = make_int4(cell, (int)p, __float_as_int(of[0]), __float_as_int(of[1]));
+        reinterpret_cast<float4 *>(r)[1] = make_float4(of[2], (float)ws[0], (float)ws[1], (float)ws[2]);
+    } else {
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) static_cast<R *>(P.off[a])[base + p] = of[a];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) static_cast<R *>(P.w[a])[base + p] = (R)ws[a];
+        P.id[base + p] = (int)p;
+    }
+}
+
+template <int DIM>
+static void load_t(int prec, cudaStream_t st, unsigned nb, int nt, long long n, const double *x0, const double *x1,
+                   const double *x2, const double *w0, const double *w1, const double *w2, int nx, int ny, int nz,
+                   const PoolBuf &P, LoadRec *rec, long long base)
+{
+    if (prec == 0)
+        k_load<double, DIM, false><<<nb, nt, 0, st>>>(n, x0, x1, x2, w0, w1, w2, nx, ny, nz, P, nullptr, base);
+    else if (rec)
+        k_load<float, DIM, true><<<nb, nt, 0, st>>>(n, x0, x1, x2, w0, w1, w2, nx, ny, nz, P, rec, base);
+    else
+        k_load<float, DIM, false><<<nb, nt, 0, st>>>(n, x0, x1, x2, w0, w1, w2, nx, ny, nz, P, nullptr, base);
 }
 
 cudaError_t launch_load(int prec, cudaStream_t st, long long n, const double *x0, const double *x1,
                         const double *x2, const double *w0, const double *w1, const double *w2, int dims, int nx,
-                        int ny, int nz, const PoolBuf &P, long long base)
+                        int ny, int nz, const PoolBuf &P, long long base, LoadRec *rec)
 {
     if (n <= 0) return cudaSuccess;
     const int nt = 256;
-    const long long nb = (n + nt - 1) / nt;
-    if (prec == 0) {
-        k_load<double><<<(unsigned)nb, nt, 0, st>>>(n, x0, x1, dims == 3 ? x2 : x0, w0, w1, w2, dims, nx, ny, nz,
-                                                    P.cell, (double *)P.off[0], (double *)P.off[1],
-                                                    dims == 3 ? (double *)P.off[2] : (double *)P.off[0],
-                                                    (double *)P.w[0], (double *)P.w[1], (double *)P.w[2], P.id, base);
-    } else {
-        k_load<float><<<(unsigned)nb, nt, 0, st>>>(n, x0, x1, dims == 3 ? x2 : x0, w0, w1, w2, dims, nx, ny, nz,
-                                                   P.cell, (float *)P.off[0], (float *)P.off[1],
-                                                   dims == 3 ? (float *)P.off[2] : (float *)P.off[0],
-                                                   (float *)P.w[0], (float *)P.w[1], (float *)P.w[2], P.id, base);
-    }
+    const unsigned nb = (unsigned)((n + nt - 1) / nt);
+    if (dims == 3)
+        load_t<3>(prec, st, nb, nt, n, x0, x1, x2, w0, w1, w2, nx, ny, nz, P, rec, base);
+    else
+        load_t<2>(prec, st, nb, nt, n, x0, x1, x2, w0, w1, w2, nx, ny, nz, P, rec, base);
+    return cudaGetLastError();
+}
+
+// A range of an FP32 pool into records, for a load that keeps other groups.
+template <int DIM>
+__global__ void k_copy_pool_rec(long long n, PoolBuf S, long long sb, int *cell, LoadRec *rec, long long db)
+{
+    const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (p >= n) return;
+    auto at = [&](void *v) { return static_cast<const float *>(v)[sb + p]; };
+    const int c = S.cell[sb + p];
+    if (cell + db != S.cell + sb) cell[db + p] = c;
+    int4 *r = reinterpret_cast<int4 *>(rec + db + p);
+    r[0] = make_int4(c, S.id[sb + p], __float_as_int(at(S.off[0])), __float_as_int(at(S.off[1])));
+    reinterpret_cast<float4 *>(r)[1] = make_float4(DIM == 3 ? at(S.off[2]) : 0.f, at(S.w[0]), at(S.w[1]), at(S.w[2]));
+}
+
+cudaError_t launch_copy_pool_rec(cudaStream_t st, const PoolBuf &src, long long sb, int *dst_cell, LoadRec *rec,
+                                 long long db, long long n, int dims)
+{
+    if (n <= 0) return cudaSuccess;
+    const int nt = 256;
+    const unsigned nb = (unsigned)((n + nt - 1) / nt);
+    if (dims == 3)
+        k_copy_pool_rec<3><<<nb, nt, 0, st>>>(n, src, sb, dst_cell, rec, db);
+    else
+        k_copy_pool_rec<2><<<nb, nt, 0, st>>>(n, src, sb, dst_cell, rec, db);
     return cudaGetLastError();
 }
 
