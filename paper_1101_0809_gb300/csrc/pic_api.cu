@@ -286,19 +286,18 @@ void graph_drop(pic_grid *g)
 // (the limit the fixed-point scales are set for), or less when a small pool's
 // items would leave SMs idle.  The 2D FP64 run of 32x32 cells and 8192 particles
 // has 16 tiles: whole, they keep 16 of the 152 SMs busy for 85 us a step; in 128
-// items of 64 particles the step takes 51 us instead of 101.  FP64 takes four items
-// per SM (one block alone leaves the FP64 pipe idle while it stages and flushes
-// its tile) of at least 64 particles (a warp's FP64 instruction takes 16 cycles,
-// so two warps hide most latencies); FP32 one per SM of at least one round of the
-// block: 256x256 cells and 2^20 particles take 2.75 ms per 40 steps in 256 whole
+// items of 64 particles the step takes 51 us instead of 101, in 256 of 32 another
+// 2 percent less.  FP64 takes eight items per SM (one block alone leaves the FP64
+// pipe idle while it stages and flushes its tile) of at least a warp; FP32 one per
+// SM of at least one round of the block: 256x256 cells and 2^20 particles take 2.75 ms per 40 steps in 256 whole
 // tiles and 2.78 ms in 768 parts.
 int item_length(const pic_grid *g, long long total)
 {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const long long slots = (long long)std::max(1, sms) * (g->prec == PIC_FP64 ? 4 : 1);
-    const long long least = std::min(g->ppi, g->prec == PIC_FP64 ? 64 : kThreads);
+    const long long slots = (long long)std::max(1, sms) * (g->prec == PIC_FP64 ? 8 : 1);
+    const long long least = std::min(g->ppi, g->prec == PIC_FP64 ? 32 : kThreads);
     const long long len = (((total + slots - 1) / slots) + 31) & ~31LL;
     return (int)std::max(least, std::min<long long>(len, g->ppi));
 }

@@ -20,6 +20,8 @@
 
 #include <cooperative_groups.h>
 
+#include <algorithm>
+
 #include "pic_internal.h"
 
 namespace cg = cooperative_groups;
@@ -47,20 +49,46 @@ struct PartArgs {
 
 extern __shared__ __align__(16) unsigned char g_smem[];
 
+// Per-warp deposit queue of particles that changed cell: capacity (a warp adds
+// at most 32 entries to fewer than 32) and the values kept per entry (old and
+// new offsets, u_z in 2D) besides one packed int (tile base << 8 | shifts + 1).
+constexpr int kQueueCap = 64;
+constexpr int kQueueVals = 7;
+
 // Blocks per SM the kernels are compiled for: two (128 registers), three of the
 // 2D FP32 ones (80).  Where the shared tiles leave room for one block only, the
-// launches take the variant compiled for one, whose registers hold everything:
-// 8x8x8 FP32 tiles and every 3D FP64 tile spilled 100 to 200 bytes per thread
-// at 128 registers (48^3 cells, 16 + 16 particles each, FP64: 5.3 -> 4.7 ms a
-// step).  The 2D FP32 persistent step of 24 runs took 22.5 ms per 30 steps at
+// launches take the variant compiled for one.  In FP32 that has 512 threads, to
+// have as many warps as two blocks would (61x47x53 cells in 8x8x8 tiles, 12 + 12
+// particles each, 20 steps: 7.76 ms with 256 threads and all registers, 6.54 with
+// 512).  In FP64 it has 256 threads whose registers hold everything: every 3D tile
+// spilled 100 to 200 bytes per thread at 128 registers (48^3 cells, 16 + 16
+// particles each: 5.3 -> 4.7 ms a step).  The 2D FP32 persistent step of 24 runs took 22.5 ms per 30 steps at
 // two blocks, 19.7 at three and 21.0 at four.
 template <int DIM, typename R>
 constexpr int min_blocks()
 {
     return DIM == 2 && sizeof(R) == 4 ? 3 : 2;
 }
+template <typename R, bool ONE>
+constexpr int block_threads()
+{
+    return ONE && sizeof(R) == 4 ? 512 : kThreads;
+}
 // The shared memory of an SM, and what the system keeps of it per block.
 inline bool one_block_per_sm(size_t smem) { return 2 * (smem + 1024) > 228 * 1024; }
+// The shared memory of a block of nt threads, given that of kThreads: more warps'
+// deposit queues and counts.
+template <typename R>
+constexpr size_t queue_bytes(int nt)
+{
+    return (size_t)(nt / 32) * (kQueueCap * (kQueueVals * sizeof(R) + sizeof(int)) + sizeof(int));
+}
+template <typename R, int MODE>
+constexpr size_t smem_of(size_t smem, int nt)
+{
+    return MODE == 1 ? smem : smem + queue_bytes<R>(nt) - queue_bytes<R>(kThreads);
+}
+constexpr size_t kSmemMax = 227 * 1024 - 16;   // less MODE 1's static word
 
 // Tile geometry of the particle kernels: extents T0 x T1 x T2, halo G and the
 // shared tiles' x and y pitches P0, P1.  GeoDyn reads them from the run and the
@@ -76,13 +104,6 @@ struct GeoFix {
     static constexpr bool dyn = false;
     static constexpr int T0 = t0, T1 = t1, T2 = t2, G = g, P0 = p0, P1 = p1;
 };
-
-
-// Per-warp deposit queue of particles that changed cell: capacity (a warp adds
-// at most 32 entries to fewer than 32) and the values kept per entry (old and
-// new offsets, u_z in 2D) besides one packed int (tile base << 8 | shifts + 1).
-constexpr int kQueueCap = 64;
-constexpr int kQueueVals = 7;
 
 __device__ __forceinline__ bool finite3(float a, float b, float c) { return isfinite(a) && isfinite(b) && isfinite(c); }
 __device__ __forceinline__ bool finite3(double a, double b, double c) { return isfinite(a) && isfinite(b) && isfinite(c); }
@@ -109,7 +130,7 @@ __device__ __forceinline__ int local_coord(int i, int o, int T, int G, int n)
 }
 
 // Where the particles of a drifted item are now: the mean displacement of
-// (up to) kThreads of them, evenly spaced over the item, from the centre of its
+// (up to) NT (threads) of them, evenly spaced over the item, from the centre of its
 // tile, in whole cells.  The item then stages the tile moved by that much.  Any
 // shift gives the same step; it only decides which particles find their stencil
 // in shared memory.  A plasma that streams or is pushed by a laser carries a
@@ -120,17 +141,17 @@ __device__ __forceinline__ int local_coord(int i, int o, int T, int G, int n)
 // steps since the sort) on the global-memory path: for the few that leave a tile
 // of a thermal plasma, which has no common drift to follow, the read cost more
 // than it gave (8x8x8 tiles, 20 steps: 8.07 -> 8.9 ms when one was enough).
-template <int DIM, typename R, bool OLD>
+template <int DIM, typename R, bool OLD, int NT>
 __device__ __forceinline__ void item_shift(const PartArgs<R> &a, const WorkItem &it, const RunDev &rn, const int T[3],
                                            int o[3])
 {
-    __shared__ int sum[4];
+    int *const sum = reinterpret_cast<int *>(g_smem);   // four words, before the tiles are staged
     if (threadIdx.x < 4) sum[threadIdx.x] = 0;
     __syncthreads();
     const long long len = it.end - it.begin;
     int d[4] = {0, 0, 0, 0};
     if (threadIdx.x < len) {
-        const long long p = it.begin + (len <= kThreads ? threadIdx.x : len * threadIdx.x / kThreads);
+        const long long p = it.begin + (len <= NT ? threadIdx.x : len * threadIdx.x / NT);
         const int cell = OLD ? a.old_cell[p] : a.P.cell[p];
         const int rest = divu31(cell, rn.div_nx);
         const int k = DIM == 3 ? divu31(rest, rn.div_ny) : 0;
@@ -152,7 +173,7 @@ __device__ __forceinline__ void item_shift(const PartArgs<R> &a, const WorkItem 
     const float w = 0.5f / (float)max(sum[3], 1);
 #pragma unroll
     for (int x = 0; x < DIM; ++x) o[x] = wrapi(o[x] + (int)rintf((float)sum[x] * w), rn.n[x]);
-    __syncthreads();
+    __syncthreads();   // the words are free for the tiles
 }
 
 // A particle past the staged tile: the same arithmetic on the periodic global
@@ -316,7 +337,7 @@ __device__ __noinline__ void far_particle(const PartArgs<R> &a, int group, long 
 // stencil only).  ORD = 4 is the comparison scheme of Eq. wrong1: its gather
 // reaches the integer points -1..2 (field tile halo (halo + 2)); its charge and
 // current are those of l_a = 1 1/2.
-template <int DIM, typename R, int MODE, class GEO, int ORD = 3, bool PERM = false>
+template <int DIM, typename R, int MODE, class GEO, int ORD = 3, bool PERM = false, int NT = kThreads>
 __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
 {
     // MODE 0 right after a sort whose arrays have not moved: the state comes
@@ -336,7 +357,7 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
     int org[3] = {tx * T0, ty * T1, tz * T2};
     if (!RP && 8LL * it.drifted > it.end - it.begin) {   // uniform over the block; none right after a sort
         const int T[3] = {T0, T1, T2};
-        item_shift<DIM, R, MODE == 2>(a, it, rn, T, org);
+        item_shift<DIM, R, MODE == 2, NT>(a, it, rn, T, org);
     }
     const int ox = org[0], oy = org[1], oz = org[2];
     constexpr int FH = ORD == 3 ? 1 : 2, JH = ORD == 5 ? 3 : 2;   // field and current halo beyond G
@@ -380,13 +401,42 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
         }
     }
 
+    // Deposit queue of this warp (MODES 0, 2).  A particle that stayed in its
+    // cell along every axis deposits at once with three-cell windows (54
+    // contributions in 3D, 21 in 2D), where its lane's bank is the one the tile
+    // sort gave it.  A particle that changed cell needs four-cell windows along
+    // the axes it crossed; it is queued and deposited later together with 31
+    // other such particles, so that the wider windows are paid only by warps
+    // of moved particles.  The integer current sums do not depend on the order.
+    // The warps' queues lie one after another (values, then codes), followed by
+    // one count per warp for the merged drain at the end of the item.
+    const int warp = threadIdx.x >> 5;
+    R *qv0 = nullptr, *qv = nullptr;
+    int *qs0 = nullptr, *qs = nullptr, *qcnt = nullptr;
+    if (NEED_J) {
+        unsigned char *qb = g_smem + (NEED_F ? 6 * (size_t)nf * sizeof(R) : 0) + (FIX ? 28 : 24) * (size_t)nj;
+        qv0 = reinterpret_cast<R *>(qb);
+        qs0 = reinterpret_cast<int *>(qb + (size_t)(NT / 32) * kQueueCap * kQueueVals * sizeof(R));
+        qcnt = qs0 + (NT / 32) * kQueueCap;
+        qv = qv0 + (size_t)warp * kQueueCap * kQueueVals;
+        qs = qs0 + warp * kQueueCap;
+    }
+
     // Particles past the staged tile: their indices in the item go to the item's
     // part of far_list, and far_particle steps them together after the others.  A
     // warp with one such lane would otherwise run the global-memory path for it
     // alone (the tenth step of item_shift's slab: 8.0 ms), and a call from inside
     // the loop would spill what the loop keeps in registers.
-    __shared__ int nfar;
-    if (threadIdx.x == 0) nfar = 0;
+    // Their number stands in a value of the queue that this dimension does not
+    // use, so that the kernels take no more shared memory for it.
+    int *nfar;
+    if constexpr (NEED_J) {
+        nfar = reinterpret_cast<int *>(qv0 + (DIM == 3 ? 6 : 2) * kQueueCap);
+    } else {
+        __shared__ int count;
+        nfar = &count;
+    }
+    if (threadIdx.x == 0) *nfar = 0;
 
     if (NEED_F) {
         // Asynchronous copies, so that all of a thread's are in flight at once, of two
@@ -456,26 +506,6 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
     }
     const R c2 = cl * cl;
 
-    // Deposit queue of this warp (MODES 0, 2).  A particle that stayed in its
-    // cell along every axis deposits at once with three-cell windows (54
-    // contributions in 3D, 21 in 2D), where its lane's bank is the one the tile
-    // sort gave it.  A particle that changed cell needs four-cell windows along
-    // the axes it crossed; it is queued and deposited later together with 31
-    // other such particles, so that the wider windows are paid only by warps
-    // of moved particles.  The integer current sums do not depend on the order.
-    // The warps' queues lie one after another (values, then codes), followed by
-    // one count per warp for the merged drain at the end of the item.
-    const int warp = threadIdx.x >> 5;
-    R *qv0 = nullptr, *qv = nullptr;
-    int *qs0 = nullptr, *qs = nullptr, *qcnt = nullptr;
-    if (NEED_J) {
-        unsigned char *qb = g_smem + (NEED_F ? 6 * (size_t)nf * sizeof(R) : 0) + (FIX ? 28 : 24) * (size_t)nj;
-        qv0 = reinterpret_cast<R *>(qb);
-        qs0 = reinterpret_cast<int *>(qb + (size_t)(kThreads / 32) * kQueueCap * kQueueVals * sizeof(R));
-        qcnt = qs0 + (kThreads / 32) * kQueueCap;
-        qv = qv0 + (size_t)warp * kQueueCap * kQueueVals;
-        qs = qs0 + warp * kQueueCap;
-    }
     const int lane = threadIdx.x & 31;
     int qn = 0;   // entries in this warp's queue (warp-uniform)
 
@@ -558,13 +588,35 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
     // RP: the permutation index of the lane's next particle is read one round ahead
     unsigned sp_next = 0;
     if (RP && it.begin + threadIdx.x < it.end) sp_next = a.perm[it.begin + threadIdx.x];
-    for (long long pw = it.begin + (threadIdx.x & ~31); pw < it.end; pw += blockDim.x) {
+    // PRE: a round's state is read while the round before is worked on.  256x256
+    // cells of 16 particles, 40 steps: 2.75 -> 2.63 ms; the 24 batched runs, 30
+    // steps: 20.2 -> 19.1 ms; 128^3 cells of 32 + 32, 12 steps: 106.2 -> 104.8 ms.
+    // Not in FP64 (18.27 ms with and without at 48^3) nor where it lost: tiles read
+    // at run time in 3D (61x47x53, 8x8x8: 6.54 -> 6.57 ms) and halos of two, whose
+    // particles are often not in the tile (slab: 17.9 -> 18.1 ms).
+    constexpr bool PRE = FIX && MODE == 0 && !RP && (DIM == 2 || (!GEO::dyn && GEO::G < 2));
+    int pre_c = 0;
+    R pre_o0 = 0, pre_o1 = 0, pre_o2 = 0, pre_w0 = 0, pre_w1 = 0, pre_w2 = 0;
+    auto fetch = [&](long long q) {
+        if (q < it.end) {
+            pre_c = a.P.cell[q];
+            pre_o0 = a.P.off[0][q];
+            pre_o1 = a.P.off[1][q];
+            if (DIM == 3) pre_o2 = a.P.off[2][q];
+            pre_w0 = a.P.w[0][q];
+            pre_w1 = a.P.w[1][q];
+            pre_w2 = a.P.w[2][q];
+        }
+    };
+    if (PRE) fetch(it.begin + threadIdx.x);
+    for (long long pw = it.begin + (threadIdx.x & ~31); pw < it.end; pw += NT) {
         const long long p = pw + lane;
         const bool valid = p < it.end;
+        const long long pn = pw + NT;   // the warp's next round
         unsigned sp_cur = 0;
         if (RP) {
             sp_cur = sp_next;
-            if (p + blockDim.x < it.end) sp_next = a.perm[p + blockDim.x];
+            if (pn + lane < it.end) sp_next = a.perm[pn + lane];
         }
         bool live = false;   // the particle moves and deposits this step
         bool far = false;    // it lies past the staged tile: far_particle steps it later
@@ -575,12 +627,17 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
             // ---- the particle's state at x^n (old) -------------------------------
             const long long sp = RP ? (long long)sp_cur : p;   // where the state is read
             const Pool<R> &src = RP ? a.S : a.P;
-            const int cell0 = MODE == 2 ? a.old_cell[p] : src.cell[sp];
-            o0 = MODE == 2 ? a.old_off[0][p] : src.off[0][sp];
-            o1 = MODE == 2 ? a.old_off[1][p] : src.off[1][sp];
-            o2 = DIM == 3 ? (MODE == 2 ? a.old_off[2][p] : src.off[2][sp]) : R(0);
+            const int cell0 = PRE ? pre_c : MODE == 2 ? a.old_cell[p] : src.cell[sp];
+            o0 = PRE ? pre_o0 : MODE == 2 ? a.old_off[0][p] : src.off[0][sp];
+            o1 = PRE ? pre_o1 : MODE == 2 ? a.old_off[1][p] : src.off[1][sp];
+            o2 = DIM == 3 ? (PRE ? pre_o2 : MODE == 2 ? a.old_off[2][p] : src.off[2][sp]) : R(0);
             R w[3] = {R(0), R(0), R(0)};
-            if (MODE != 2 || DIM == 2) {
+            if (PRE) {
+                w[0] = pre_w0;
+                w[1] = pre_w1;
+                w[2] = pre_w2;
+                fetch(pn + lane);
+            } else if (MODE != 2 || DIM == 2) {
                 w[0] = src.w[0][sp];
                 w[1] = src.w[1][sp];
                 w[2] = src.w[2][sp];
@@ -706,7 +763,7 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
         const unsigned fm = __ballot_sync(0xffffffffu, far);
         if (fm != 0u) {   // warp-uniform
             int at = 0;
-            if (lane == 0) at = atomicAdd(&nfar, __popc(fm));
+            if (lane == 0) at = atomicAdd(nfar, __popc(fm));
             at = __shfl_sync(0xffffffffu, at, 0) + __popc(fm & ((1u << lane) - 1u));
             if (far) a.far_list[it.begin + at] = (unsigned)(p - it.begin);
         }
@@ -797,14 +854,15 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
     }
     if (NEED_J && lane == 0) qcnt[warp] = qn;
     __syncthreads();
-    if (nfar > 0) {
-        for (int m = threadIdx.x; m < nfar; m += blockDim.x) {
+    const int nf_all = *nfar;
+    if (nf_all > 0) {
+        for (int m = threadIdx.x; m < nf_all; m += blockDim.x) {
             const long long pf = it.begin + a.far_list[it.begin + m];
             far_particle<DIM, R, MODE, ORD, RP>(a, it.group, pf, RP ? (long long)a.perm[pf] : pf);
         }
         if (MODE != 2 && threadIdx.x == 0) {   // the sort policy's measure of drift, and item_shift's
-            atomicAdd(reinterpret_cast<unsigned *>(a.err) + 1, (unsigned)nfar);
-            a.items[item].drifted = it.drifted + nfar;
+            atomicAdd(reinterpret_cast<unsigned *>(a.err) + 1, (unsigned)nf_all);
+            a.items[item].drifted = it.drifted + nf_all;
         }
     }
     if (NEED_J) {
@@ -815,11 +873,11 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
         // partly filled drain per item instead of one per warp.
         int tot = 0;
 #pragma unroll
-        for (int w = 0; w < kThreads / 32; ++w) tot += qcnt[w];
+        for (int w = 0; w < NT / 32; ++w) tot += qcnt[w];
         for (int m0 = threadIdx.x & ~31; m0 < tot; m0 += blockDim.x) {   // uniform over the warp
             int src = 0, slot = m0 + lane;
 #pragma unroll
-            for (int w = 0; w < kThreads / 32 - 1; ++w) {
+            for (int w = 0; w < NT / 32 - 1; ++w) {
                 const int c = qcnt[src];
                 if (slot >= c) {
                     slot -= c;
@@ -977,10 +1035,11 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
 }
 
 template <int DIM, typename R, int MODE, class GEO = GeoDyn, int ORD = 3, bool PERM = false, bool ONE = false>
-__global__ void __launch_bounds__(kThreads, ONE ? 1 : min_blocks<DIM, R>()) k_particles(const __grid_constant__ PartArgs<R> a)
+__global__ void __launch_bounds__(block_threads<R, ONE>(), ONE ? 1 : min_blocks<DIM, R>())
+    k_particles(const __grid_constant__ PartArgs<R> a)
 {
     if ((int)blockIdx.x >= *a.n_items) return;
-    process_item<DIM, R, MODE, GEO, ORD, PERM>(a, blockIdx.x);
+    process_item<DIM, R, MODE, GEO, ORD, PERM, block_threads<R, ONE>()>(a, blockIdx.x);
 }
 
 // Run of a batch that owns concatenated cell l (run_cell_base has nruns + 1 entries).
@@ -1037,20 +1096,27 @@ template <int DIM, typename R, int MODE, class GEO = GeoDyn, int ORD = 3>
 static cudaError_t launch_t(cudaStream_t st, int max_items, size_t smem, const PartArgs<R> &a)
 {
     if (max_items <= 0) return cudaSuccess;
-    constexpr bool both = GEO::dyn && DIM == 3;
-    if constexpr (MODE == 0 && ORD == 3) {
-        if (a.perm) {   // right after a sort: the kernel that reads through the permutation
-            if (both && one_block_per_sm(smem))
-                k_particles<DIM, R, 0, GEO, 3, true, both><<<max_items, kThreads, smem, st>>>(a);
-            else
-                k_particles<DIM, R, 0, GEO, 3, true><<<max_items, kThreads, smem, st>>>(a);
+    if constexpr (GEO::dyn && DIM == 3) {
+        constexpr int nt = block_threads<R, true>();
+        const size_t smem1 = smem_of<R, MODE>(smem, nt);
+        if (one_block_per_sm(smem) && smem1 <= kSmemMax) {
+            if constexpr (MODE == 0 && ORD == 3) {
+                if (a.perm) {
+                    k_particles<DIM, R, 0, GEO, 3, true, true><<<max_items, nt, smem1, st>>>(a);
+                    return cudaGetLastError();
+                }
+            }
+            k_particles<DIM, R, MODE, GEO, ORD, false, true><<<max_items, nt, smem1, st>>>(a);
             return cudaGetLastError();
         }
     }
-    if (both && one_block_per_sm(smem))
-        k_particles<DIM, R, MODE, GEO, ORD, false, both><<<max_items, kThreads, smem, st>>>(a);
-    else
-        k_particles<DIM, R, MODE, GEO, ORD><<<max_items, kThreads, smem, st>>>(a);
+    if constexpr (MODE == 0 && ORD == 3) {
+        if (a.perm) {   // right after a sort: the kernel that reads through the permutation
+            k_particles<DIM, R, 0, GEO, 3, true><<<max_items, kThreads, smem, st>>>(a);
+            return cudaGetLastError();
+        }
+    }
+    k_particles<DIM, R, MODE, GEO, ORD><<<max_items, kThreads, smem, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -1062,8 +1128,9 @@ static cudaError_t set_limit_one(int bytes)
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if constexpr (GEO::dyn && DIM == 3) {
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_particles<DIM, R, MODE, GEO, ORD, PERM, true>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+            e = cudaFuncSetAttribute(
+                k_particles<DIM, R, MODE, GEO, ORD, PERM, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                (int)std::min(kSmemMax, smem_of<R, MODE>((size_t)bytes, block_threads<R, true>())));
     }
     return e;
 }
