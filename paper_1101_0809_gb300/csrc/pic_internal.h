@@ -80,6 +80,11 @@ cudaError_t launch_load(int prec, cudaStream_t st, long long n, const double *x0
 cudaError_t launch_yee(int prec, int which, int zero_j, cudaStream_t st, const RunDev *runs, int nruns,
                        long long max_cells, void *const E[3], void *const B[3], void *const J[3], int dims,
                        const long long *ant_n);
+// The second B half step and the E step of a step in one pass: E and B go to E1
+// and B1, other buffers.
+cudaError_t launch_yee_b_half_e(int dims, int prec, cudaStream_t st, const RunDev *runs, int nruns,
+                                long long max_cells, void *const E[3], void *const B[3], void *const J[3],
+                                void *const E1[3], void *const B1[3], const long long *ant_n);
 // Advances every run's antenna clock (E steps since its antenna was set) by one.
 cudaError_t launch_antenna_tick(cudaStream_t st, long long *ant_n, int nruns);
 
@@ -225,6 +230,13 @@ struct pic_grid {
     void *E[3] = {nullptr, nullptr, nullptr};
     void *B[3] = {nullptr, nullptr, nullptr};
     void *J[3] = {nullptr, nullptr, nullptr};
+    // the buffers that the pass of the second B half step and the E step writes, swapped
+    // with E and B then; null when there was no memory for them (the step then
+    // takes two passes in place)
+    void *E1[3] = {nullptr, nullptr, nullptr};
+    void *B1[3] = {nullptr, nullptr, nullptr};
+    void *EB1 = nullptr;            // their one allocation
+    bool in_EB1 = false;            // E and B are in it now (an odd number of swaps)
 
     // species / groups
     std::vector<pic::HostGroup> groups;
