@@ -21,6 +21,8 @@ constexpr int kSortItems = 16;
 constexpr int kChunk = kSortThreads * kSortItems;   // keys per chunk
 constexpr int kScanItems = 8;
 constexpr int kScanSeg = kSortThreads * kScanItems; // elements per scan block
+constexpr int kItemsThreads = 1024;     // threads of the one-block kernels over tiles
+constexpr int kItemsOneBlock = 4096;    // tiles up to which they are taken
 
 // ---------------------------------------------------------------------------
 // Exclusive scan of unsigned counts: per-block sums, one block scanning the
@@ -816,6 +818,27 @@ __global__ void k_resort_newcnt(int n, unsigned *stay, const unsigned *mstart, c
     mbef[t] = aft[t] == 0xffffffffu ? movin : aft[t] - mstart[t];
 }
 
+// The same and its exclusive scan in one block, for few tiles.
+__global__ void __launch_bounds__(kItemsThreads) k_resort_newcnt_one(int n, unsigned *stay, const unsigned *mstart,
+                                                                    const unsigned *aft, unsigned *mbef)
+{
+    __shared__ unsigned wt[32];
+    unsigned before = 0;
+    for (int t0 = 0; t0 < n; t0 += kItemsThreads) {
+        const int t = t0 + threadIdx.x;
+        unsigned c = 0;
+        if (t < n) {
+            const unsigned movin = t + 1 < n ? mstart[t + 1] - mstart[t] : 0u;
+            c = stay[t] + movin;
+            mbef[t] = aft[t] == 0xffffffffu ? movin : aft[t] - mstart[t];
+        }
+        unsigned all;
+        const unsigned at = before + block_exclusive_scan(c, wt, all);
+        if (t < n) stay[t] = at;
+        before += all;
+    }
+}
+
 __global__ void k_resort_tile_start(int n, const unsigned *nst, long long *tile_start)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1070,6 +1093,60 @@ __global__ void k_tile_start(const unsigned *keys, long long n, int total_tiles,
         for (long long t = k + 1; t <= total_tiles; ++t) tile_start[t] = n;
 }
 
+// The work items of one tile: [b, e) in parts of at most ppi particles, equal
+// and of whole warps, to items[s ..].  part <= ppi (a multiple of 32), so that
+// part * (cnt - 1) <= ppi * (cnt - 1) < e - b and no item is empty.
+__device__ __forceinline__ void tile_items(int t, long long b, long long e, int cnt, int ppi, const GroupDev *groups,
+                                           int ngroups, WorkItem *items)
+{
+    if (cnt <= 0) return;
+    const int part = (int)((((e - b + cnt - 1) / cnt) + 31) & ~31LL);
+    int lo = 0, hi = ngroups;
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (groups[mid].tile_base <= t) lo = mid; else hi = mid;
+    }
+    for (int q = 0; q < cnt; ++q) {
+        WorkItem w;
+        w.group = lo;
+        w.tile = t - groups[lo].tile_base;
+        w.begin = b + (long long)q * part;
+        w.end = w.begin + part < e ? w.begin + part : e;
+        w.drifted = 0;
+        items[q] = w;
+    }
+}
+
+// All of it in one block, for few tiles: counts, their scan and the items, and
+// before that the tile starts of a re-sort (nst, else null).  Six launches of 2.5
+// to 3.5 us each otherwise (three for a restored snapshot), longer than the work.
+__global__ void __launch_bounds__(kItemsThreads) k_items_one(const unsigned *nst, long long *tile_start,
+                                                             int total_tiles, int ppi, const GroupDev *groups,
+                                                             int ngroups, WorkItem *items, int *n_items)
+{
+    __shared__ unsigned wt[32];
+    unsigned before = 0;
+    for (int t0 = 0; t0 <= total_tiles; t0 += kItemsThreads) {   // uniform over the block
+        const int t = t0 + threadIdx.x;
+        long long b = 0, e = 0;
+        if (nst && t <= total_tiles) tile_start[t] = b = nst[t];
+        if (t < total_tiles) {
+            if (nst) {
+                e = nst[t + 1];
+            } else {
+                b = tile_start[t];
+                e = tile_start[t + 1];
+            }
+        }
+        const unsigned cnt = t < total_tiles ? (unsigned)((e - b + ppi - 1) / ppi) : 0u;
+        unsigned all;
+        const unsigned at = before + block_exclusive_scan(cnt, wt, all);
+        tile_items(t, b, e, (int)cnt, ppi, groups, ngroups, items + at);
+        before += all;
+    }
+    if (threadIdx.x == 0) *n_items = (int)before;
+}
+
 __global__ void k_item_counts(const long long *tile_start, int total_tiles, int ppi, unsigned *counts)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1085,24 +1162,8 @@ __global__ void k_items(const long long *tile_start, const unsigned *scan, int t
     if (t >= total_tiles) return;
     const long long b = tile_start[t], e = tile_start[t + 1];
     const int cnt = (int)((e - b + ppi - 1) / ppi);
-    // equal parts, in whole warps: part <= ppi (a multiple of 32), so that
-    // part * (cnt - 1) <= ppi * (cnt - 1) < e - b and no item is empty
-    const int part = cnt > 0 ? (int)((((e - b + cnt - 1) / cnt) + 31) & ~31LL) : ppi;
-    int lo = 0, hi = ngroups;
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (groups[mid].tile_base <= t) lo = mid; else hi = mid;
-    }
     const unsigned s = scan[t];
-    for (int q = 0; q < cnt; ++q) {
-        WorkItem w;
-        w.group = lo;
-        w.tile = t - groups[lo].tile_base;
-        w.begin = b + (long long)q * part;
-        w.end = w.begin + part < e ? w.begin + part : e;
-        w.drifted = 0;
-        items[s + q] = w;
-    }
+    tile_items(t, b, e, cnt, ppi, groups, ngroups, items + s);
     if (t == total_tiles - 1) *n_items = (int)(s + cnt);
 }
 
@@ -1248,10 +1309,16 @@ cudaError_t sort_and_build_items(int prec, int dims, cudaStream_t st, long long 
                                                                                               mstart, aft);
         *launches += 1;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        k_resort_newcnt<<<nbt, nt, 0, st>>>(ntp, stay, mstart, aft, mbef);
-        *launches += 1;
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        if ((e = exclusive_scan(stay, ntp, scr.block_sums, st, launches)) != cudaSuccess) return e;
+        if (ntp <= kItemsOneBlock) {
+            k_resort_newcnt_one<<<1, kItemsThreads, 0, st>>>(ntp, stay, mstart, aft, mbef);
+            *launches += 1;
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        } else {
+            k_resort_newcnt<<<nbt, nt, 0, st>>>(ntp, stay, mstart, aft, mbef);
+            *launches += 1;
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+            if ((e = exclusive_scan(stay, ntp, scr.block_sums, st, launches)) != cudaSuccess) return e;
+        }
         k_resort_order<<<(unsigned)total_tiles, kSortThreads, 0, st>>>(tile_start, total, stay, mstart, mbef,
                                                                        scr.vals[cur], scr.cls, src.cell, groups,
                                                                        ngroups, runs, rule, scr.vals[1 - cur]);
@@ -1262,6 +1329,12 @@ cudaError_t sort_and_build_items(int prec, int dims, cudaStream_t st, long long 
         } else {
             if ((e = launch_permute4(prec, dims, st, total, src, dst, scr.vals[1 - cur])) != cudaSuccess) return e;
             *launches += 1;
+        }
+        if (ntp <= kItemsOneBlock) {
+            k_items_one<<<1, kItemsThreads, 0, st>>>(stay, tile_start, total_tiles, particles_per_item, groups,
+                                                     ngroups, items, n_items);
+            *launches += 1;
+            return cudaGetLastError();
         }
         k_resort_tile_start<<<nbt, nt, 0, st>>>(ntp, stay, tile_start);
         *launches += 1;
@@ -1348,6 +1421,12 @@ cudaError_t build_items(cudaStream_t st, const long long *tile_start, int total_
                         const GroupDev *groups, int ngroups, SortScratch &scr, unsigned *item_scan, WorkItem *items,
                         int *n_items, int *launches)
 {
+    if (total_tiles <= kItemsOneBlock) {
+        k_items_one<<<1, kItemsThreads, 0, st>>>(nullptr, const_cast<long long *>(tile_start), total_tiles,
+                                                 particles_per_item, groups, ngroups, items, n_items);
+        *launches += 1;
+        return cudaGetLastError();
+    }
     cudaError_t e;
     const int nt = 256;
     const unsigned nbt = (unsigned)((total_tiles + nt - 1) / nt);
