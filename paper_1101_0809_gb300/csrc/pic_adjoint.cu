@@ -585,42 +585,33 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? 2 : 1) k_particles_
             sLo[c] = q + (6 + c) * nf;
         }
     }
-    for (int l = threadIdx.x; l < nf; l += blockDim.x) {
-        if constexpr (FIX) {
+    // the tiles as in process_item: asynchronous copies, and 16-byte clears
+    auto stage = [&](R *const *dst, const R *const *src, int h, int e0, int e1, int e2) {
+        for (int q = threadIdx.x; q < e0 * e1 * e2; q += blockDim.x) {
+            const int lx = q % e0, r = q / e0, ly = r % e1, lz = r / e1;
+            const int gx = wrapi(ox - h + lx, nx), gy = wrapi(oy - h + ly, ny);
+            const int gz = DIM == 3 ? wrapi(oz - h + lz, nz) : 0;
+            const long long gi = cb + gx + (long long)nx * (gy + (long long)ny * gz);
+            const int l = lx + P0 * (ly + P1 * lz);
 #pragma unroll
-            for (int c = 0; c < 6; ++c) {
-                sH[c][l] = 0;
-                sLo[c][l] = 0;
-            }
-        } else {
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                sLE[c][l] = R(0);
-                sLB[c][l] = R(0);
-            }
+            for (int c = 0; c < 3; ++c) copy_async<sizeof(R)>(dst[c] + l, src[c] + gi);
         }
-        const int lx = l % P0, r = l / P0, ly = r % P1, lz = r / P1;
-        if (lx >= fe0 || ly >= fe1) continue;   // pitch padding
-        const int gx = wrapi(ox - G - 1 + lx, nx);
-        const int gy = wrapi(oy - G - 1 + ly, ny);
-        const int gz = DIM == 3 ? wrapi(oz - G - 1 + lz, nz) : 0;
-        const long long gi = cb + gx + (long long)nx * (gy + (long long)ny * gz);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            sE[c][l] = a.E[c][gi];
-            sB[c][l] = a.B1[c][gi];
+    };
+    stage(sE, a.E, G + 1, fe0, fe1, fe2);
+    stage(sB, a.B1, G + 1, fe0, fe1, fe2);
+    stage(sL, a.lamJ, G + 2, je0, je1, je2);
+    {
+        // lambda tiles: 12 * nf words in FP32, 6 * nf doubles in FP64
+        int *z = reinterpret_cast<int *>(reinterpret_cast<R *>(g_smem) + 6 * nf);
+        const int nw = 12 * nf;
+        int l0 = 0;
+        if ((nf & 1) == 0) {
+            for (int l = threadIdx.x; l < nw >> 2; l += blockDim.x) reinterpret_cast<int4 *>(z)[l] = make_int4(0, 0, 0, 0);
+            l0 = nw & ~3;
         }
+        for (int l = l0 + threadIdx.x; l < nw; l += blockDim.x) z[l] = 0;
     }
-    for (int l = threadIdx.x; l < nj; l += blockDim.x) {
-        const int lx = l % P0, r = l / P0, ly = r % P1, lz = r / P1;
-        if (lx >= je0 || ly >= je1) continue;
-        const int gx = wrapi(ox - G - 2 + lx, nx);
-        const int gy = wrapi(oy - G - 2 + ly, ny);
-        const int gz = DIM == 3 ? wrapi(oz - G - 2 + lz, nz) : 0;
-        const long long gi = cb + gx + (long long)nx * (gy + (long long)ny * gz);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) sL[c][l] = a.lamJ[c][gi];
-    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     // FP32: the fixed-point scale, 2^(33 - ceil(log2 bound)) for lambdas up to
     // bound = 256 x the previous launch's largest (a work item holds at most
     // 8192 particles, so every word's sum stays within 2^46); none yet: every
@@ -842,8 +833,15 @@ static cudaError_t adj_part_t(cudaStream_t st, const AdjLaunch &lc, const PoolBu
     a.lam_cur = lc.lam_cur;
     if (lc.total <= 0) return cudaSuccess;
     if (lc.items && lc.max_items > 0) {
-        // blocks per work item: about 512 particles or more per block on average
-        long long ns = lc.total / ((long long)lc.max_items * 512);
+        // blocks per work item: as many as give every SM two, of about 512 particles
+        // or more on average.  A block's tiles (18 staged or cleared, 12 flushed)
+        // cost more than its share of the particles gains once the chip is full: 256
+        // items of 4096 particles, 40 steps of the differentiable run: 13.5 ms in
+        // five blocks per item, 13.25 in two, 13.0 in one.
+        int dev = 0, sms = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        const long long ns = std::min(lc.total / ((long long)lc.max_items * 512), 2LL * sms / lc.max_items);
         const int nsplit = (int)(ns < 1 ? 1 : ns > 8 ? 8 : ns);
         const size_t smem = adjoint_smem_bytes(DIM, sizeof(R) == 8 ? 0 : 1, lc.tile, lc.halo, lc.pitch);
         k_particles_adj_tiled<DIM, R><<<(unsigned)((long long)lc.max_items * nsplit), kThreads, smem, st>>>(

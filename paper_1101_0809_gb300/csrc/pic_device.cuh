@@ -102,6 +102,16 @@ struct Fields {
 
 enum : int { ERR_NONFINITE = 1 };
 
+// 4, 8 or 16 bytes from global to shared memory, both aligned to as much,
+// without waiting; complete after cp.async.wait_all of the thread.
+template <int BYTES>
+__device__ __forceinline__ void copy_async(void *dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+                 "n"(BYTES)
+                 : "memory");
+}
+
 __device__ __forceinline__ int wrapi(int i, int n)
 {
     return i < 0 ? i + n : (i >= n ? i - n : i);

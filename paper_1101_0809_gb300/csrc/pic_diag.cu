@@ -189,8 +189,10 @@ struct GlobalZeroB5 {   // offsets -2..2 from the l_a = 2 1/2 base index
 // ORD = 5 (l_a = 2 1/2): E and rho tiles with a halo of (halo + 2) cells, the
 // 4-cell cubic weights around the base index.  ORD = 4 (Eq. wrong1): the same
 // halo for its gather, the l_a = 1 1/2 charge.
+// Three blocks per SM, at the price of spills (96^3 cells of 8 + 8 particles: a step
+// pass with diagnostics 5.69 ms, 5.79 at two blocks without spills).
 template <int DIM, int ORD = 3>
-__global__ void __launch_bounds__(kDiagThreads, 2) k_diag_items(int run, const WorkItem *items, const int *n_items,
+__global__ void __launch_bounds__(kDiagThreads, 3) k_diag_items(int run, const WorkItem *items, const int *n_items,
                                                              const GroupDev *groups, const RunDev *runs, Pool<float> P,
                                                              Fields<float> F, int halo, double *rho, double *partials)
 {
@@ -211,6 +213,7 @@ __global__ void __launch_bounds__(kDiagThreads, 2) k_diag_items(int run, const W
     int *rl = rh + nf;
     const long long cb = rn.cell_base;
     const float cl = rn.cf, c2 = cl * cl;
+    const DivU31 div_nx = rn.div_nx, div_ny = rn.div_ny;
     for (int item = blockIdx.x; item < ni; item += gridDim.x) {
         const WorkItem it = items[item];
         const GroupDev &gr = groups[it.group];
@@ -219,17 +222,19 @@ __global__ void __launch_bounds__(kDiagThreads, 2) k_diag_items(int run, const W
         const int ty = (it.tile / rn.ntile[0]) % rn.ntile[1];
         const int tz = DIM == 3 ? it.tile / (rn.ntile[0] * rn.ntile[1]) : 0;
         const int ox = tx * T0, oy = ty * T1, oz = tz * T2;
-        for (int l = threadIdx.x; l < nf; l += blockDim.x) {
-            const int lx = l % P0, r = l / P0, ly = r % P1, lz = r / P1;
-            rh[l] = 0;
-            rl[l] = 0;
-            if (lx >= fe0 || ly >= fe1) continue;   // pitch padding
+        // the tile as in the particle kernels: asynchronous copies of the used cells
+        for (int q = threadIdx.x; q < fe0 * fe1 * fe2; q += blockDim.x) {
+            const int lx = q % fe0, r = q / fe0, ly = r % fe1, lz = r / fe1;
             const int gx = wrapi(ox - G - FH + lx, nx);
             const int gy = wrapi(oy - G - FH + ly, ny);
             const int gz = DIM == 3 ? wrapi(oz - G - FH + lz, nz) : 0;
             const long long gi = cb + gx + (long long)nx * (gy + (long long)ny * gz);
-            for (int c = 0; c < 3; ++c) sE[c][l] = F.E[c][gi];
+            const int l = lx + P0 * (ly + P1 * lz);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) copy_async<4>(sE[c] + l, F.E[c] + gi);
         }
+        for (int l = threadIdx.x; l < 2 * nf; l += blockDim.x) rh[l] = 0;
+        asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
         const float qV = (float)(gr.qp / rn.V);
         const float kq = qV * gr.rscale;
@@ -252,9 +257,9 @@ __global__ void __launch_bounds__(kDiagThreads, 2) k_diag_items(int run, const W
         };
         for (long long p = it.begin + threadIdx.x; p < it.end; p += blockDim.x) {
             const int c0 = P.cell[p];
-            const int rest = divu31(c0, rn.div_nx);
+            const int rest = divu31(c0, div_nx);
             const int i = c0 - rest * nx;
-            const int k = DIM == 3 ? divu31(rest, rn.div_ny) : 0;
+            const int k = DIM == 3 ? divu31(rest, div_ny) : 0;
             const int j = rest - k * ny;
             int li = i - ox, lj = j - oy, lk = k - oz;
             if (li >= T0 + G) li -= nx; if (li < -G) li += nx;
@@ -395,23 +400,25 @@ __global__ void __launch_bounds__(kDiagThreads) k_diag_cells(const RunDev *runs,
     const long long ncell = (long long)nx * ny * nz;
     const long long stride = (long long)gridDim.x * blockDim.x;
     const double hx = 0.5 * rn.cN[0], hy = 0.5 * rn.cN[1], hz = 0.5 * rn.cN[2];
+    // the FP64 pipe bounds this kernel: reciprocals of the cell sizes instead of three
+    // quotients per cell
+    const double id0 = 1.0 / rn.d[0], id1 = 1.0 / rn.d[1], id2 = 1.0 / rn.d[2];
     for (long long l = blockIdx.x * (long long)blockDim.x + threadIdx.x; l < ncell; l += stride) {
-        const int i = (int)(l % nx);
-        const long long r = l / nx;
-        const int j = (int)(r % ny), k = (int)(r / ny);
+        int i, j, k;
+        yee_ijk(rn, (int)l, i, j, k);
         const long long p = rn.cell_base + l;
         const long long pip = p + (i == nx - 1 ? -(nx - 1) : 1), pim = p + (i == 0 ? nx - 1 : -1);
         const long long pjp = p + (long long)nx * (j == ny - 1 ? -(ny - 1) : 1);
         const long long pjm = p + (long long)nx * (j == 0 ? ny - 1 : -1);
         const double ex = F.E[0][p], ey = F.E[1][p], ez = F.E[2][p];
-        double div = ((double)F.E[0][pip] - ex) / rn.d[0] + ((double)F.E[1][pjp] - ey) / rn.d[1];
+        double div = ((double)F.E[0][pip] - ex) * id0 + ((double)F.E[1][pjp] - ey) * id1;
         double bx = (double)F.B[0][p] - hy * (ez - (double)F.E[2][pjm]);
         double by = (double)F.B[1][p] + hx * (ez - (double)F.E[2][pim]);
         double bz = (double)F.B[2][p] - hx * (ey - (double)F.E[1][pim]) + hy * (ex - (double)F.E[0][pjm]);
         if (DIM == 3) {
             const long long pkp = p + (long long)nx * ny * (k == nz - 1 ? -(nz - 1) : 1);
             const long long pkm = p + (long long)nx * ny * (k == 0 ? nz - 1 : -1);
-            div += ((double)F.E[2][pkp] - ez) / rn.d[2];
+            div += ((double)F.E[2][pkp] - ez) * id2;
             bx += hz * (ey - (double)F.E[1][pkm]);
             by -= hz * (ex - (double)F.E[0][pkm]);
         }

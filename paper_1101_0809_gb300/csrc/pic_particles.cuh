@@ -108,16 +108,6 @@ struct GeoFix {
 __device__ __forceinline__ bool finite3(float a, float b, float c) { return isfinite(a) && isfinite(b) && isfinite(c); }
 __device__ __forceinline__ bool finite3(double a, double b, double c) { return isfinite(a) && isfinite(b) && isfinite(c); }
 
-// 4, 8 or 16 bytes from global to shared memory, both aligned to as much,
-// without waiting; complete after cp.async.wait_all of the thread.
-template <int BYTES>
-__device__ __forceinline__ void copy_async(void *dst, const void *src)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
-                 "n"(BYTES)
-                 : "memory");
-}
-
 // Tile-local coordinate of global index i for a tile starting at o with extent T:
 // the periodic image in [-G, T+G) if there is one (the grid is wider than the
 // staged region, so at most one image lies there), else a value outside it.
