@@ -491,85 +491,98 @@ struct GlobalAcc {
 // its third face only the closure sum of Pm (zero up to rounding; the window
 // of an unshifted particle has two interior faces), and those contributions are
 // skipped.  The flag is warp-uniform, so the skip is a uniform branch.
+// only (warp-uniform): the one component to deposit, or -1 for all three.
 template <int DIM, typename R, class Acc>
 __device__ __forceinline__ void deposit(const Acc &acc, const AxisWin<R> &X, const AxisWin<R> &Y, const AxisWin<R> &Z,
-                                        const R kf[3], R uz, int full)
+                                        const R kf[3], R uz, int full, int only = -1)
 {
     const R third = R(1) / R(3);
     const bool fx = full & 1, fy = full & 2, fz = full & 4;
     if (DIM == 3) {
+        if (only < 0 || only == 0) {
 #pragma unroll
-        for (int wz = 0; wz < 4; ++wz) {
-            if (wz == 3 && !fz) continue;
+            for (int wz = 0; wz < 4; ++wz) {
+                if (wz == 3 && !fz) continue;
+#pragma unroll
+                for (int wy = 0; wy < 4; ++wy) {
+                    if (wy == 3 && !fy) continue;
+                    const R T = Y.Pp[wy] * Z.Pp[wz] + third * Y.Pm[wy] * Z.Pm[wz];
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) {
+                        if (q == 2 && !fx) continue;
+                        acc.add(0, X.lo + 1 + q, Y.lo + wy, Z.lo + wz, kf[0] * X.D[q], T);
+                    }
+                }
+            }
+        }
+        if (only < 0 || only == 1) {
+#pragma unroll
+            for (int wz = 0; wz < 4; ++wz) {
+                if (wz == 3 && !fz) continue;
+#pragma unroll
+                for (int wx = 0; wx < 4; ++wx) {
+                    if (wx == 3 && !fx) continue;
+                    const R T = X.Pp[wx] * Z.Pp[wz] + third * X.Pm[wx] * Z.Pm[wz];
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) {
+                        if (q == 2 && !fy) continue;
+                        acc.add(1, X.lo + wx, Y.lo + 1 + q, Z.lo + wz, kf[1] * Y.D[q], T);
+                    }
+                }
+            }
+        }
+        if (only < 0 || only == 2) {
 #pragma unroll
             for (int wy = 0; wy < 4; ++wy) {
                 if (wy == 3 && !fy) continue;
-                const R T = Y.Pp[wy] * Z.Pp[wz] + third * Y.Pm[wy] * Z.Pm[wz];
 #pragma unroll
-                for (int q = 0; q < 3; ++q) {
-                    if (q == 2 && !fx) continue;
-                    acc.add(0, X.lo + 1 + q, Y.lo + wy, Z.lo + wz, kf[0] * X.D[q], T);
-                }
-            }
-        }
+                for (int wx = 0; wx < 4; ++wx) {
+                    if (wx == 3 && !fx) continue;
+                    const R T = X.Pp[wx] * Y.Pp[wy] + third * X.Pm[wx] * Y.Pm[wy];
 #pragma unroll
-        for (int wz = 0; wz < 4; ++wz) {
-            if (wz == 3 && !fz) continue;
-#pragma unroll
-            for (int wx = 0; wx < 4; ++wx) {
-                if (wx == 3 && !fx) continue;
-                const R T = X.Pp[wx] * Z.Pp[wz] + third * X.Pm[wx] * Z.Pm[wz];
-#pragma unroll
-                for (int q = 0; q < 3; ++q) {
-                    if (q == 2 && !fy) continue;
-                    acc.add(1, X.lo + wx, Y.lo + 1 + q, Z.lo + wz, kf[1] * Y.D[q], T);
-                }
-            }
-        }
-#pragma unroll
-        for (int wy = 0; wy < 4; ++wy) {
-            if (wy == 3 && !fy) continue;
-#pragma unroll
-            for (int wx = 0; wx < 4; ++wx) {
-                if (wx == 3 && !fx) continue;
-                const R T = X.Pp[wx] * Y.Pp[wy] + third * X.Pm[wx] * Y.Pm[wy];
-#pragma unroll
-                for (int q = 0; q < 3; ++q) {
-                    if (q == 2 && !fz) continue;
-                    acc.add(2, X.lo + wx, Y.lo + wy, Z.lo + 1 + q, kf[2] * Z.D[q], T);
+                    for (int q = 0; q < 3; ++q) {
+                        if (q == 2 && !fz) continue;
+                        acc.add(2, X.lo + wx, Y.lo + wy, Z.lo + 1 + q, kf[2] * Z.D[q], T);
+                    }
                 }
             }
         }
     } else {
+        if (only < 0 || only == 0) {
 #pragma unroll
-        for (int wy = 0; wy < 4; ++wy) {
-            if (wy == 3 && !fy) continue;
-            const R t = kf[0] * Y.Pp[wy];
+            for (int wy = 0; wy < 4; ++wy) {
+                if (wy == 3 && !fy) continue;
+                const R t = kf[0] * Y.Pp[wy];
 #pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                if (q == 2 && !fx) continue;
-                acc.add(0, X.lo + 1 + q, Y.lo + wy, 0, t, X.D[q]);
+                for (int q = 0; q < 3; ++q) {
+                    if (q == 2 && !fx) continue;
+                    acc.add(0, X.lo + 1 + q, Y.lo + wy, 0, t, X.D[q]);
+                }
             }
         }
-#pragma unroll
-        for (int wx = 0; wx < 4; ++wx) {
-            if (wx == 3 && !fx) continue;
-            const R t = kf[1] * X.Pp[wx];
-#pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                if (q == 2 && !fy) continue;
-                acc.add(1, X.lo + wx, Y.lo + 1 + q, 0, t, Y.D[q]);
-            }
-        }
-        const R kz = kf[2] * uz;
-#pragma unroll
-        for (int wy = 0; wy < 4; ++wy) {
-            if (wy == 3 && !fy) continue;
+        if (only < 0 || only == 1) {
 #pragma unroll
             for (int wx = 0; wx < 4; ++wx) {
                 if (wx == 3 && !fx) continue;
-                const R T = X.Pp[wx] * Y.Pp[wy] + third * X.Pm[wx] * Y.Pm[wy];
-                acc.add(2, X.lo + wx, Y.lo + wy, 0, kz, T);
+                const R t = kf[1] * X.Pp[wx];
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    if (q == 2 && !fy) continue;
+                    acc.add(1, X.lo + wx, Y.lo + 1 + q, 0, t, Y.D[q]);
+                }
+            }
+        }
+        const R kz = kf[2] * uz;
+        if (only < 0 || only == 2) {
+#pragma unroll
+            for (int wy = 0; wy < 4; ++wy) {
+                if (wy == 3 && !fy) continue;
+#pragma unroll
+                for (int wx = 0; wx < 4; ++wx) {
+                    if (wx == 3 && !fx) continue;
+                    const R T = X.Pp[wx] * Y.Pp[wy] + third * X.Pm[wx] * Y.Pm[wy];
+                    acc.add(2, X.lo + wx, Y.lo + wy, 0, kz, T);
+                }
             }
         }
     }
@@ -779,83 +792,95 @@ __device__ __forceinline__ void axis_window5(R d0, R d1, int s, AxisWin5<R> &a)
 // fourth face (the closure) are skipped.
 template <int DIM, typename R, class Acc>
 __device__ __forceinline__ void deposit5(const Acc &acc, const AxisWin5<R> &X, const AxisWin5<R> &Y,
-                                         const AxisWin5<R> &Z, const R kf[3], R uz, int full)
+                                         const AxisWin5<R> &Z, const R kf[3], R uz, int full, int only = -1)
 {
     const R third = R(1) / R(3);
     const bool fx = full & 1, fy = full & 2, fz = full & 4;
     if (DIM == 3) {
+        if (only < 0 || only == 0) {
 #pragma unroll
-        for (int wz = 0; wz < 5; ++wz) {
-            if (wz == 4 && !fz) continue;
+            for (int wz = 0; wz < 5; ++wz) {
+                if (wz == 4 && !fz) continue;
+#pragma unroll
+                for (int wy = 0; wy < 5; ++wy) {
+                    if (wy == 4 && !fy) continue;
+                    const R T = Y.Pp[wy] * Z.Pp[wz] + third * Y.Pm[wy] * Z.Pm[wz];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        if (q == 3 && !fx) continue;
+                        acc.add(0, X.lo + 1 + q, Y.lo + wy, Z.lo + wz, kf[0] * X.D[q], T);
+                    }
+                }
+            }
+        }
+        if (only < 0 || only == 1) {
+#pragma unroll
+            for (int wz = 0; wz < 5; ++wz) {
+                if (wz == 4 && !fz) continue;
+#pragma unroll
+                for (int wx = 0; wx < 5; ++wx) {
+                    if (wx == 4 && !fx) continue;
+                    const R T = X.Pp[wx] * Z.Pp[wz] + third * X.Pm[wx] * Z.Pm[wz];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        if (q == 3 && !fy) continue;
+                        acc.add(1, X.lo + wx, Y.lo + 1 + q, Z.lo + wz, kf[1] * Y.D[q], T);
+                    }
+                }
+            }
+        }
+        if (only < 0 || only == 2) {
 #pragma unroll
             for (int wy = 0; wy < 5; ++wy) {
                 if (wy == 4 && !fy) continue;
-                const R T = Y.Pp[wy] * Z.Pp[wz] + third * Y.Pm[wy] * Z.Pm[wz];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    if (q == 3 && !fx) continue;
-                    acc.add(0, X.lo + 1 + q, Y.lo + wy, Z.lo + wz, kf[0] * X.D[q], T);
-                }
-            }
-        }
+                for (int wx = 0; wx < 5; ++wx) {
+                    if (wx == 4 && !fx) continue;
+                    const R T = X.Pp[wx] * Y.Pp[wy] + third * X.Pm[wx] * Y.Pm[wy];
 #pragma unroll
-        for (int wz = 0; wz < 5; ++wz) {
-            if (wz == 4 && !fz) continue;
-#pragma unroll
-            for (int wx = 0; wx < 5; ++wx) {
-                if (wx == 4 && !fx) continue;
-                const R T = X.Pp[wx] * Z.Pp[wz] + third * X.Pm[wx] * Z.Pm[wz];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    if (q == 3 && !fy) continue;
-                    acc.add(1, X.lo + wx, Y.lo + 1 + q, Z.lo + wz, kf[1] * Y.D[q], T);
-                }
-            }
-        }
-#pragma unroll
-        for (int wy = 0; wy < 5; ++wy) {
-            if (wy == 4 && !fy) continue;
-#pragma unroll
-            for (int wx = 0; wx < 5; ++wx) {
-                if (wx == 4 && !fx) continue;
-                const R T = X.Pp[wx] * Y.Pp[wy] + third * X.Pm[wx] * Y.Pm[wy];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    if (q == 3 && !fz) continue;
-                    acc.add(2, X.lo + wx, Y.lo + wy, Z.lo + 1 + q, kf[2] * Z.D[q], T);
+                    for (int q = 0; q < 4; ++q) {
+                        if (q == 3 && !fz) continue;
+                        acc.add(2, X.lo + wx, Y.lo + wy, Z.lo + 1 + q, kf[2] * Z.D[q], T);
+                    }
                 }
             }
         }
     } else {
+        if (only < 0 || only == 0) {
 #pragma unroll
-        for (int wy = 0; wy < 5; ++wy) {
-            if (wy == 4 && !fy) continue;
-            const R t = kf[0] * Y.Pp[wy];
+            for (int wy = 0; wy < 5; ++wy) {
+                if (wy == 4 && !fy) continue;
+                const R t = kf[0] * Y.Pp[wy];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                if (q == 3 && !fx) continue;
-                acc.add(0, X.lo + 1 + q, Y.lo + wy, 0, t, X.D[q]);
+                for (int q = 0; q < 4; ++q) {
+                    if (q == 3 && !fx) continue;
+                    acc.add(0, X.lo + 1 + q, Y.lo + wy, 0, t, X.D[q]);
+                }
             }
         }
-#pragma unroll
-        for (int wx = 0; wx < 5; ++wx) {
-            if (wx == 4 && !fx) continue;
-            const R t = kf[1] * X.Pp[wx];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                if (q == 3 && !fy) continue;
-                acc.add(1, X.lo + wx, Y.lo + 1 + q, 0, t, Y.D[q]);
-            }
-        }
-        const R kz = kf[2] * uz;
-#pragma unroll
-        for (int wy = 0; wy < 5; ++wy) {
-            if (wy == 4 && !fy) continue;
+        if (only < 0 || only == 1) {
 #pragma unroll
             for (int wx = 0; wx < 5; ++wx) {
                 if (wx == 4 && !fx) continue;
-                const R T = X.Pp[wx] * Y.Pp[wy] + third * X.Pm[wx] * Y.Pm[wy];
-                acc.add(2, X.lo + wx, Y.lo + wy, 0, kz, T);
+                const R t = kf[1] * X.Pp[wx];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (q == 3 && !fy) continue;
+                    acc.add(1, X.lo + wx, Y.lo + 1 + q, 0, t, Y.D[q]);
+                }
+            }
+        }
+        const R kz = kf[2] * uz;
+        if (only < 0 || only == 2) {
+#pragma unroll
+            for (int wy = 0; wy < 5; ++wy) {
+                if (wy == 4 && !fy) continue;
+#pragma unroll
+                for (int wx = 0; wx < 5; ++wx) {
+                    if (wx == 4 && !fx) continue;
+                    const R T = X.Pp[wx] * Y.Pp[wy] + third * X.Pm[wx] * Y.Pm[wy];
+                    acc.add(2, X.lo + wx, Y.lo + wy, 0, kz, T);
+                }
             }
         }
     }

@@ -501,44 +501,45 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
 
 
     auto deposit_local = [&](int base, const AxisWin<R> &X, const AxisWin<R> &Y, const AxisWin<R> &Z, R uz,
-                             int full) {
+                             int full, int only) {
         if constexpr (FIX) {
             FixedAcc acc;   // bias taken off per contribution (variable stencil)
             for (int c = 0; c < 3; ++c) { acc.hi[c] = sJh[c]; acc.lo[c] = sJl[c]; }
             acc.base = base;
             acc.s1 = P0;
             acc.s2 = P0 * P1;
-            deposit<DIM>(acc, X, Y, Z, kfs, uz, full);
+            deposit<DIM>(acc, X, Y, Z, kfs, uz, full, only);
         } else {
             SmemAcc<R> acc;
             for (int c = 0; c < 3; ++c) acc.J[c] = sJ[c];
             acc.base = base;
             acc.s1 = P0;
             acc.s2 = P0 * P1;
-            deposit<DIM>(acc, X, Y, Z, kf, uz, full);
+            deposit<DIM>(acc, X, Y, Z, kf, uz, full, only);
         }
     };
     auto deposit_local5 = [&](int base, const AxisWin5<R> &X, const AxisWin5<R> &Y, const AxisWin5<R> &Z, R uz,
-                              int full) {
+                              int full, int only) {
         if constexpr (FIX) {
             FixedAcc acc;
             for (int c = 0; c < 3; ++c) { acc.hi[c] = sJh[c]; acc.lo[c] = sJl[c]; }
             acc.base = base;
             acc.s1 = P0;
             acc.s2 = P0 * P1;
-            deposit5<DIM>(acc, X, Y, Z, kfs, uz, full);
+            deposit5<DIM>(acc, X, Y, Z, kfs, uz, full, only);
         } else {
             SmemAcc<R> acc;
             for (int c = 0; c < 3; ++c) acc.J[c] = sJ[c];
             acc.base = base;
             acc.s1 = P0;
             acc.s2 = P0 * P1;
-            deposit5<DIM>(acc, X, Y, Z, kf, uz, full);
+            deposit5<DIM>(acc, X, Y, Z, kf, uz, full, only);
         }
     };
     // deposits, on each lane with `on`, entry `slot` of the queue whose values
-    // and codes start at sv and ss (a whole warp calls it)
-    auto drain = [&](const R *sv, const int *ss, int slot, bool on) {
+    // and codes start at sv and ss (a whole warp calls it): all of its current, or
+    // the component `only` (warp-uniform)
+    auto drain = [&](const R *sv, const int *ss, int slot, bool on, int only) {
         R d0 = R(0), d1 = R(0), d2 = R(0), e0 = R(0), e1 = R(0), e2 = R(0), u = R(0);
         int code = 1 | (1 << 2) | (1 << 4);
         if (on) {
@@ -563,13 +564,13 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
                 axis_window5(d0, e0, q0, X);
                 axis_window5(d1, e1, q1, Y);
                 if (DIM == 3) axis_window5(d2, e2, q2, Z); else Z = X;
-                deposit_local5(code >> 8, X, Y, Z, u, full);
+                deposit_local5(code >> 8, X, Y, Z, u, full, only);
             } else {
                 AxisWin<R> X, Y, Z;
                 axis_window(d0, e0, q0, X);
                 axis_window(d1, e1, q1, Y);
                 if (DIM == 3) axis_window(d2, e2, q2, Z); else Z = X;
-                deposit_local(code >> 8, X, Y, Z, u, full);
+                deposit_local(code >> 8, X, Y, Z, u, full, only);
             }
         }
     };
@@ -797,7 +798,7 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
                     deposit5<DIM>(acc, X, Y, Z, kfs, uz, 0);
                     atomicAdd(&scnt[base], 1);
                 } else {
-                    deposit_local5(base, X, Y, Z, uz, 0);
+                    deposit_local5(base, X, Y, Z, uz, 0, -1);
                 }
             } else {
                 AxisWin<R> X, Y, Z;
@@ -814,7 +815,7 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
                     deposit<DIM>(acc, X, Y, Z, kfs, uz, 0);
                     atomicAdd(&scnt[base], 1);
                 } else {
-                    deposit_local(base, X, Y, Z, uz, 0);
+                    deposit_local(base, X, Y, Z, uz, 0, -1);
                 }
             }
         }
@@ -838,7 +839,7 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
         if (qn >= 32) {   // warp-uniform
             __syncwarp();
             qn -= 32;
-            drain(qv, qs, qn + lane, true);
+            drain(qv, qs, qn + lane, true, -1);
             __syncwarp();   // the drained slots are free again
         }
     }
@@ -858,13 +859,21 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
     if (NEED_J) {
         // The entries left in the warps' queues (fewer than 32 each) are drained
         // together: merged entry m is slot m - (entries of the warps before) of
-        // its warp's queue, and warp w deposits the merged entries
-        // [32w, 32w + 32), [32w + 256, ...).  A block then runs about one
-        // partly filled drain per item instead of one per warp.
+        // its warp's queue, 32 of them per drain.  While they are few, each drain is
+        // three, one per component of the current, on three warps: the block waits
+        // for the longest, and a drain of all three components is as long as
+        // a round of particles.  Few is one in FP32 (64^3 cells of 2 + 2 particles, 20
+        // steps, 4.05 -> 3.94 ms; with up to five drains in thirds the slab lost 4.6
+        // percent to forming the windows three times) and, in FP64, as many as give
+        // a warp two thirds (32x32 cells, 50 steps, 2.27 -> 2.18 ms; 48^3 of 16 + 16, 4
+        // steps, 18.24 -> 18.00).
         int tot = 0;
 #pragma unroll
         for (int w = 0; w < NT / 32; ++w) tot += qcnt[w];
-        for (int m0 = threadIdx.x & ~31; m0 < tot; m0 += blockDim.x) {   // uniform over the warp
+        const int nd = (tot + 31) >> 5;
+        const bool thirds = FIX ? nd <= 1 : 3 * nd <= 2 * (NT / 32);
+        for (int d = warp; d < (thirds ? 3 * nd : nd); d += NT / 32) {   // uniform over the warp
+            const int m0 = 32 * (thirds ? d / 3 : d);
             int src = 0, slot = m0 + lane;
 #pragma unroll
             for (int w = 0; w < NT / 32 - 1; ++w) {
@@ -876,7 +885,7 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
             }
             const bool on = m0 + lane < tot;
             drain(qv0 + (size_t)(on ? src : 0) * kQueueCap * kQueueVals, qs0 + (on ? src : 0) * kQueueCap,
-                  on ? slot : 0, on);
+                  on ? slot : 0, on, thirds ? d % 3 : -1);
         }
         __syncthreads();
         const float jinv = gr.jinv;
