@@ -329,7 +329,7 @@ __global__ void __launch_bounds__(kDiagThreads, 3) k_diag_items(int run, const W
                     if constexpr (ORD == 4)
                         gather_w1<DIM>(rd, Sx, Sy, Sz, Ep, Bp);
                     else
-                        gather<DIM>(rd, fx, Sx, fy, Sy, fz, Sz, Ep, Bp);
+                        gather<DIM, false>(rd, fx, Sx, fy, Sy, fz, Sz, Ep, Bp);
                     acc.base = rd.base;
                     const int kz0 = DIM == 3 ? -1 : 0, kz1 = DIM == 3 ? 1 : 0;
 #pragma unroll
@@ -351,7 +351,7 @@ __global__ void __launch_bounds__(kDiagThreads, 3) k_diag_items(int run, const W
                     if constexpr (ORD == 4)
                         gather_w1<DIM>(rd, Sx, Sy, Sz, Ep, Bp);
                     else
-                        gather<DIM>(rd, fx, Sx, fy, Sy, fz, Sz, Ep, Bp);
+                        gather<DIM, false>(rd, fx, Sx, fy, Sy, fz, Sz, Ep, Bp);
                     const int kz0 = DIM == 3 ? -1 : 0, kz1 = DIM == 3 ? 1 : 0;
                     for (int dz = kz0; dz <= kz1; ++dz)
                         for (int dy = -1; dy <= 1; ++dy)
