@@ -1055,6 +1055,54 @@ __device__ __forceinline__ void deposit5(const Acc &acc, const AxisWin5<R> &X, c
 }
 
 // ---------------------------------------------------------------------------
+// 3D deposit (l_a = 1 1/2) of a particle whose cell moved along one axis only,
+// written for that axis, A, and the two after it, B and C, so that the lanes of a
+// warp may hold different axes: strides, prefactors and component arrays are the
+// lane's.  B and C have three cells and two faces, A four and three: 75
+// contributions instead of 144.  J[c]: the component along A, B, C; b0: the first
+// cell of all three windows; s: strides.  only: as for deposit().
+// ---------------------------------------------------------------------------
+template <typename R>
+__device__ __forceinline__ void deposit_one_axis(R *const J[3], const AxisWin<R> &A, const AxisWin<R> &B,
+                                                 const AxisWin<R> &C, const R kf[3], int b0, const int s[3], int only)
+{
+    const R third = R(1) / R(3);
+    if (only < 0 || only == 0) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+#pragma unroll
+            for (int b = 0; b < 3; ++b) {
+                const R T = B.Pp[b] * C.Pp[c] + third * B.Pm[b] * C.Pm[c];
+#pragma unroll
+                for (int q = 0; q < 3; ++q)
+                    atomicAdd(J[0] + b0 + (1 + q) * s[0] + b * s[1] + c * s[2], kf[0] * A.D[q] * T);
+            }
+    }
+    if (only < 0 || only == 1) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                const R T = A.Pp[a] * C.Pp[c] + third * A.Pm[a] * C.Pm[c];
+#pragma unroll
+                for (int q = 0; q < 2; ++q)
+                    atomicAdd(J[1] + b0 + a * s[0] + (1 + q) * s[1] + c * s[2], kf[1] * B.D[q] * T);
+            }
+    }
+    if (only < 0 || only == 2) {
+#pragma unroll
+        for (int b = 0; b < 3; ++b)
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                const R T = A.Pp[a] * B.Pp[b] + third * A.Pm[a] * B.Pm[b];
+#pragma unroll
+                for (int q = 0; q < 2; ++q)
+                    atomicAdd(J[2] + b0 + a * s[0] + b * s[1] + (1 + q) * s[2], kf[2] * C.D[q] * T);
+            }
+    }
+}
+
+// ---------------------------------------------------------------------------
 // Yee updates of one cell l of run rn (Appendix, Eqs. updateB and escheme,
 // completed cyclically; in 2D every z difference vanishes).
 //   B half step:  Bx[i,j,k] -= (c_y/2)(Ez[i,j,k]-Ez[i,j-1,k]) - (c_z/2)(Ey[i,j,k]-Ey[i,j,k-1])

@@ -42,6 +42,7 @@ struct PartArgs {
     Fields<R> F;
     int *old_cell;
     R *old_off[3];
+    int qcap;             // entries of a warp's deposit queue in 3D FP64 (else kQueueCap)
     unsigned *far_list;   // pool-sized scratch: particles past their item's staged tile (process_item)
     int halo;
     int *err;   // err[0]: error word; err[1]: particles that ran past their tile's halo (counted by MODES 0, 1)
@@ -54,6 +55,8 @@ extern __shared__ __align__(16) unsigned char g_smem[];
 // new offsets, u_z in 2D) besides one packed int (tile base << 8 | shifts + 1).
 constexpr int kQueueCap = 64;
 constexpr int kQueueVals = 7;
+// 3D FP64: room for both kinds of particles that moved, fewer than 32 of each and 32 new
+constexpr int kQueueCap3 = 96;
 
 // Blocks per SM the kernels are compiled for: two (128 registers), three of the
 // 2D FP32 ones (80).  Where the shared tiles leave room for one block only, the
@@ -76,6 +79,7 @@ constexpr int block_threads()
 }
 // The shared memory of an SM, and what the system keeps of it per block.
 inline bool one_block_per_sm(size_t smem) { return 2 * (smem + 1024) > 228 * 1024; }
+inline int blocks_per_sm(size_t smem) { return (int)(228 * 1024 / (smem + 1024)); }
 // The shared memory of a block of nt threads, given that of kThreads: more warps'
 // deposit queues and counts.
 template <typename R>
@@ -87,6 +91,13 @@ template <typename R, int MODE>
 constexpr size_t smem_of(size_t smem, int nt)
 {
     return MODE == 1 ? smem : smem + queue_bytes<R>(nt) - queue_bytes<R>(kThreads);
+}
+// What the larger queues of 3D FP64 take more; the launches take them where they
+// neither cost a block per SM nor pass the limit.
+template <typename R>
+constexpr size_t queue3_bytes(int nt)
+{
+    return (size_t)(nt / 32) * ((kQueueCap3 - kQueueCap) * (kQueueVals * sizeof(R) + sizeof(int)) + sizeof(int));
 }
 constexpr size_t kSmemMax = 227 * 1024 - 16;   // less MODE 1's static word
 
@@ -401,15 +412,25 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
     // The warps' queues lie one after another (values, then codes), followed by
     // one count per warp for the merged drain at the end of the item.
     const int warp = threadIdx.x >> 5;
+    // In 3D FP64, where the queue has room for it (kQueueCap3), the particles that
+    // crossed one axis only, most of those that moved, are queued apart, from the
+    // queue's start, and drained with the windows they need (deposit_one_axis); the
+    // others from its end.  48^3 cells of 16 + 16 particles, 4 steps: 18.0 -> 17.4 ms.
+    // In FP32 the second drain cost the loop more registers than it gave: 128^3, 12
+    // steps, 100.8 -> 103.8 ms.
+    constexpr bool SPLIT = DIM == 3 && !FIX && ORD != 5 && NEED_J;
+    const int QC = SPLIT ? a.qcap : kQueueCap;
+    const bool split = SPLIT && QC == kQueueCap3;
     R *qv0 = nullptr, *qv = nullptr;
-    int *qs0 = nullptr, *qs = nullptr, *qcnt = nullptr;
+    int *qs0 = nullptr, *qs = nullptr, *qcnt = nullptr, *qcnt1 = nullptr;
     if (NEED_J) {
         unsigned char *qb = g_smem + (NEED_F ? 6 * (size_t)nf * sizeof(R) : 0) + (FIX ? 28 : 24) * (size_t)nj;
         qv0 = reinterpret_cast<R *>(qb);
-        qs0 = reinterpret_cast<int *>(qb + (size_t)(NT / 32) * kQueueCap * kQueueVals * sizeof(R));
-        qcnt = qs0 + (NT / 32) * kQueueCap;
-        qv = qv0 + (size_t)warp * kQueueCap * kQueueVals;
-        qs = qs0 + warp * kQueueCap;
+        qs0 = reinterpret_cast<int *>(qb + (size_t)(NT / 32) * QC * kQueueVals * sizeof(R));
+        qcnt = qs0 + (NT / 32) * QC;
+        qcnt1 = qcnt + NT / 32;   // with split
+        qv = qv0 + (size_t)warp * QC * kQueueVals;
+        qs = qs0 + warp * QC;
     }
 
     // Particles past the staged tile: their indices in the item go to the item's
@@ -421,7 +442,7 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
     // use, so that the kernels take no more shared memory for it.
     int *nfar;
     if constexpr (NEED_J) {
-        nfar = reinterpret_cast<int *>(qv0 + (DIM == 3 ? 6 : 2) * kQueueCap);
+        nfar = reinterpret_cast<int *>(qv0 + (DIM == 3 ? 6 : 2) * QC);
     } else {
         __shared__ int count;
         nfar = &count;
@@ -497,7 +518,8 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
     const R c2 = cl * cl;
 
     const int lane = threadIdx.x & 31;
-    int qn = 0;   // entries in this warp's queue (warp-uniform)
+    int qn = 0;   // entries in this warp's queue (warp-uniform): at its start, or with split at its end
+    int q1 = 0;   // with split: entries at its start
 
 
     auto deposit_local = [&](int base, const AxisWin<R> &X, const AxisWin<R> &Y, const AxisWin<R> &Z, R uz,
@@ -543,15 +565,15 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
         R d0 = R(0), d1 = R(0), d2 = R(0), e0 = R(0), e1 = R(0), e2 = R(0), u = R(0);
         int code = 1 | (1 << 2) | (1 << 4);
         if (on) {
-            d0 = sv[0 * kQueueCap + slot];
-            d1 = sv[1 * kQueueCap + slot];
-            e0 = sv[3 * kQueueCap + slot];
-            e1 = sv[4 * kQueueCap + slot];
+            d0 = sv[0 * QC + slot];
+            d1 = sv[1 * QC + slot];
+            e0 = sv[3 * QC + slot];
+            e1 = sv[4 * QC + slot];
             if (DIM == 3) {
-                d2 = sv[2 * kQueueCap + slot];
-                e2 = sv[5 * kQueueCap + slot];
+                d2 = sv[2 * QC + slot];
+                e2 = sv[5 * QC + slot];
             } else {
-                u = sv[6 * kQueueCap + slot];
+                u = sv[6 * QC + slot];
             }
             code = ss[slot];
         }
@@ -574,6 +596,25 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
             }
         }
     };
+    // the same for entries that crossed one axis
+    auto drain_one = [&](const R *sv, const int *ss, int slot, bool on, int only) {
+        if constexpr (SPLIT) {
+            if (!on) return;
+            const int code = ss[slot];
+            const int A = (code & 3) != 1 ? 0 : ((code >> 2) & 3) != 1 ? 1 : 2;
+            const int B = A == 2 ? 0 : A + 1, Cx = A == 0 ? 2 : A - 1;
+            auto of = [](int ax, auto v0, auto v1, auto v2) { return ax == 0 ? v0 : ax == 1 ? v1 : v2; };
+            const int s[3] = {of(A, 1, P0, P0 * P1), of(B, 1, P0, P0 * P1), of(Cx, 1, P0, P0 * P1)};
+            const R k[3] = {of(A, kfs[0], kfs[1], kfs[2]), of(B, kfs[0], kfs[1], kfs[2]),
+                            of(Cx, kfs[0], kfs[1], kfs[2])};
+            R *const J[3] = {sJ[0] + A * nj, sJ[0] + B * nj, sJ[0] + Cx * nj};
+            AxisWin<R> X, Y, Z;
+            axis_window(sv[A * QC + slot], sv[(3 + A) * QC + slot], ((code >> (2 * A)) & 3) - 1, X);
+            axis_window_still(sv[B * QC + slot], sv[(3 + B) * QC + slot], Y);
+            axis_window_still(sv[Cx * QC + slot], sv[(3 + Cx) * QC + slot], Z);
+            deposit_one_axis<R>(J, X, Y, Z, k, (code >> 8) + X.lo * s[0] - s[1] - s[2], s, only);
+        }
+    };
 
     // warps run whole rounds of 32 consecutive particles (the last one partial)
     // RP: the permutation index of the lane's next particle is read one round ahead
@@ -584,19 +625,25 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
     // steps: 20.2 -> 19.1 ms; 128^3 cells of 32 + 32, 12 steps: 106.2 -> 104.8 ms.
     // Not in FP64 (18.27 ms with and without at 48^3) nor where it lost: tiles read
     // at run time in 3D (61x47x53, 8x8x8: 6.54 -> 6.57 ms) and halos of two, whose
-    // particles are often not in the tile (slab: 17.9 -> 18.1 ms).
-    constexpr bool PRE = FIX && MODE == 0 && !RP && (DIM == 2 || (!GEO::dyn && GEO::G < 2));
-    int pre_c = 0;
+    // particles are often not in the tile (slab: 17.9 -> 18.1 ms).  Through a sort's
+    // permutation in 2D only (the batched runs 18.2 -> 18.0 ms; 128^3 103.3 -> 103.8).
+    constexpr bool PRE = FIX && MODE == 0 && (DIM == 2 || (!RP && !GEO::dyn && GEO::G < 2));
+    int pre_c = 0, pre_id = 0;
+    unsigned sp_after = 0;   // RP with PRE: the permutation index of the round after next
+    if (PRE && RP && it.begin + NT + threadIdx.x < it.end) sp_after = a.perm[it.begin + NT + threadIdx.x];
     R pre_o0 = 0, pre_o1 = 0, pre_o2 = 0, pre_w0 = 0, pre_w1 = 0, pre_w2 = 0;
     auto fetch = [&](long long q) {
         if (q < it.end) {
-            pre_c = a.P.cell[q];
-            pre_o0 = a.P.off[0][q];
-            pre_o1 = a.P.off[1][q];
-            if (DIM == 3) pre_o2 = a.P.off[2][q];
-            pre_w0 = a.P.w[0][q];
-            pre_w1 = a.P.w[1][q];
-            pre_w2 = a.P.w[2][q];
+            const Pool<R> &src = RP ? a.S : a.P;
+            const long long sq = RP ? (long long)sp_next : q;
+            pre_c = src.cell[sq];
+            pre_o0 = src.off[0][sq];
+            pre_o1 = src.off[1][sq];
+            if (DIM == 3) pre_o2 = src.off[2][sq];
+            pre_w0 = src.w[0][sq];
+            pre_w1 = src.w[1][sq];
+            pre_w2 = src.w[2][sq];
+            if (RP) pre_id = src.id[sq];
         }
     };
     if (PRE) fetch(it.begin + threadIdx.x);
@@ -607,13 +654,18 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
         unsigned sp_cur = 0;
         if (RP) {
             sp_cur = sp_next;
-            if (pn + lane < it.end) sp_next = a.perm[pn + lane];
+            if (PRE) {
+                sp_next = sp_after;
+                if (pn + NT + lane < it.end) sp_after = a.perm[pn + NT + lane];
+            } else if (pn + lane < it.end) {
+                sp_next = a.perm[pn + lane];
+            }
         }
         bool live = false;   // the particle moves and deposits this step
         bool far = false;    // it lies past the staged tile: far_particle steps it later
         int i = 0, j = 0, k = 0, li = 0, lj = 0, lk = 0;
         R o0 = R(0), o1 = R(0), o2 = R(0), n0 = R(0), n1 = R(0), n2 = R(0), uz = R(0);
-        int s0 = 0, s1 = 0, s2 = 0;
+        int s0 = 0, s1 = 0, s2 = 0, id = 0;
         if (valid) {
             // ---- the particle's state at x^n (old) -------------------------------
             const long long sp = RP ? (long long)sp_cur : p;   // where the state is read
@@ -627,6 +679,7 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
                 w[0] = pre_w0;
                 w[1] = pre_w1;
                 w[2] = pre_w2;
+                id = pre_id;
                 fetch(pn + lane);
             } else if (MODE != 2 || DIM == 2) {
                 w[0] = src.w[0][sp];
@@ -702,7 +755,7 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
                     atomicOr(a.err, ERR_NONFINITE);
                     live = false;   // the particle keeps x^n and contributes no current
                     if (RP) {   // ... in its slot of the new order, with the momentum it reached
-                        a.P.id[p] = a.S.id[sp];
+                        a.P.id[p] = PRE ? id : a.S.id[sp];
                         a.P.cell[p] = cell0;
                         a.P.off[0][p] = o0;
                         a.P.off[1][p] = o1;
@@ -723,7 +776,7 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
                         a.old_off[1][p] = o1;
                         if (DIM == 3) a.old_off[2][p] = o2;
                     }
-                    if (RP) a.P.id[p] = a.S.id[sp];   // the id moves with the particle
+                    if (RP) a.P.id[p] = PRE ? id : a.S.id[sp];   // the id moves with the particle
                     a.P.cell[p] = cell1;
                     a.P.off[0][p] = n0;
                     a.P.off[1][p] = n1;
@@ -765,7 +818,7 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
         // l_a = 1 1/2 the offsets and cell shifts themselves; for l_a = 2 1/2 the
         // base index is cell + (offset >= 1/2), so it moves with the cell shift
         // and the half-offset flags.
-        int q0 = s0, q1 = s1, q2 = s2;
+        int q0 = s0, qy = s1, q2 = s2;
         R a0 = o0, a1 = o1, a2 = o2, b0 = n0, b1 = n1, b2 = n2;
         int ub0 = 0, ub1 = 0, ub2 = 0;   // old base index - old cell
         if constexpr (ORD == 5) {
@@ -773,13 +826,13 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
             ub1 = split5(o1, a1);
             const int v0 = split5(n0, b0), v1 = split5(n1, b1);
             q0 = s0 + v0 - ub0;
-            q1 = s1 + v1 - ub1;
+            qy = s1 + v1 - ub1;
             if (DIM == 3) {
                 ub2 = split5(o2, a2);
                 q2 = s2 + split5(n2, b2) - ub2;
             }
         }
-        const bool moved = (q0 | q1 | q2) != 0;
+        const bool moved = (q0 | qy | q2) != 0;
         const int base = (li + ub0 + G + JH) +
                          P0 * ((lj + ub1 + G + JH) + (DIM == 3 ? P1 * (lk + ub2 + G + JH) : 0));
         if (live && !moved) {
@@ -821,29 +874,44 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
         }
         const bool enq = live && moved;
         const unsigned qm = __ballot_sync(0xffffffffu, enq);
+        const bool one = split && enq && (q0 != 0) + (qy != 0) + (q2 != 0) == 1;
+        const unsigned om = split ? __ballot_sync(0xffffffffu, one) : 0u;
+        const unsigned mm = qm & ~om;
         if (enq) {
-            const int slot = qn + __popc(qm & ((1u << lane) - 1u));
-            qv[0 * kQueueCap + slot] = a0;
-            qv[1 * kQueueCap + slot] = a1;
-            qv[3 * kQueueCap + slot] = b0;
-            qv[4 * kQueueCap + slot] = b1;
+            const unsigned below = (1u << lane) - 1u;
+            const int slot = one ? q1 + __popc(om & below)
+                                 : split ? QC - 1 - (qn + __popc(mm & below)) : qn + __popc(mm & below);
+            qv[0 * QC + slot] = a0;
+            qv[1 * QC + slot] = a1;
+            qv[3 * QC + slot] = b0;
+            qv[4 * QC + slot] = b1;
             if (DIM == 3) {
-                qv[2 * kQueueCap + slot] = a2;
-                qv[5 * kQueueCap + slot] = b2;
+                qv[2 * QC + slot] = a2;
+                qv[5 * QC + slot] = b2;
             } else {
-                qv[6 * kQueueCap + slot] = uz;
+                qv[6 * QC + slot] = uz;
             }
-            qs[slot] = (base << 8) | (q0 + 1) | ((q1 + 1) << 2) | ((q2 + 1) << 4);
+            qs[slot] = (base << 8) | (q0 + 1) | ((qy + 1) << 2) | ((q2 + 1) << 4);
         }
-        qn += __popc(qm);
+        qn += __popc(mm);
+        q1 += __popc(om);
         if (qn >= 32) {   // warp-uniform
             __syncwarp();
             qn -= 32;
-            drain(qv, qs, qn + lane, true, -1);
+            drain(qv, qs, split ? QC - 1 - (qn + lane) : qn + lane, true, -1);
             __syncwarp();   // the drained slots are free again
         }
+        if (q1 >= 32) {   // warp-uniform
+            __syncwarp();
+            q1 -= 32;
+            drain_one(qv, qs, q1 + lane, true, -1);
+            __syncwarp();
+        }
     }
-    if (NEED_J && lane == 0) qcnt[warp] = qn;
+    if (NEED_J && lane == 0) {
+        qcnt[warp] = qn;
+        if (split) qcnt1[warp] = q1;
+    }
     __syncthreads();
     const int nf_all = *nfar;
     if (nf_all > 0) {
@@ -867,25 +935,36 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
         // percent to forming the windows three times) and, in FP64, as many as give
         // a warp two thirds (32x32 cells, 50 steps, 2.27 -> 2.18 ms; 48^3 of 16 + 16, 4
         // steps, 18.24 -> 18.00).
-        int tot = 0;
+        int tot = 0, tot1 = 0;
 #pragma unroll
-        for (int w = 0; w < NT / 32; ++w) tot += qcnt[w];
-        const int nd = (tot + 31) >> 5;
+        for (int w = 0; w < NT / 32; ++w) {
+            tot += qcnt[w];
+            if (split) tot1 += qcnt1[w];
+        }
+        const int nd1 = (tot1 + 31) >> 5, nd = nd1 + ((tot + 31) >> 5);
         const bool thirds = FIX ? nd <= 1 : 3 * nd <= 2 * (NT / 32);
         for (int d = warp; d < (thirds ? 3 * nd : nd); d += NT / 32) {   // uniform over the warp
-            const int m0 = 32 * (thirds ? d / 3 : d);
-            int src = 0, slot = m0 + lane;
+            const int which = thirds ? d / 3 : d, only = thirds ? d % 3 : -1;
+            const bool one = which < nd1;
+            const int *cnt = one ? qcnt1 : qcnt;
+            const int m = 32 * (one ? which : which - nd1) + lane;
+            const bool on = m < (one ? tot1 : tot);
+            int src = 0, slot = m;
 #pragma unroll
             for (int w = 0; w < NT / 32 - 1; ++w) {
-                const int c = qcnt[src];
+                const int c = cnt[src];
                 if (slot >= c) {
                     slot -= c;
                     ++src;
                 }
             }
-            const bool on = m0 + lane < tot;
-            drain(qv0 + (size_t)(on ? src : 0) * kQueueCap * kQueueVals, qs0 + (on ? src : 0) * kQueueCap,
-                  on ? slot : 0, on, thirds ? d % 3 : -1);
+            if (!on) src = slot = 0;
+            const R *sv = qv0 + (size_t)src * QC * kQueueVals;
+            const int *ss = qs0 + src * QC;
+            if (one)
+                drain_one(sv, ss, slot, on, only);
+            else
+                drain(sv, ss, split ? QC - 1 - slot : slot, on, only);
         }
         __syncthreads();
         const float jinv = gr.jinv;
@@ -1091,14 +1170,27 @@ __global__ void __launch_bounds__(kThreads, ONE ? 1 : min_blocks<DIM, R>()) k_st
     }
 }
 
+// The launch's deposit queues: their capacity, and the shared memory they add to smem.
+template <int DIM, typename R, int MODE>
+static size_t choose_queue(size_t smem, int nt, int *qcap)
+{
+    *qcap = kQueueCap;
+    if (DIM != 3 || sizeof(R) == 4 || MODE == 1) return smem;
+    const size_t more = smem + queue3_bytes<R>(nt);
+    if (more > kSmemMax || std::min(2, blocks_per_sm(more)) < std::min(2, blocks_per_sm(smem))) return smem;
+    *qcap = kQueueCap3;
+    return more;
+}
+
 template <int DIM, typename R, int MODE, class GEO = GeoDyn, int ORD = 3>
-static cudaError_t launch_t(cudaStream_t st, int max_items, size_t smem, const PartArgs<R> &a)
+static cudaError_t launch_t(cudaStream_t st, int max_items, size_t smem, PartArgs<R> a)
 {
     if (max_items <= 0) return cudaSuccess;
     if constexpr (GEO::dyn && DIM == 3) {
         constexpr int nt = block_threads<R, true>();
-        const size_t smem1 = smem_of<R, MODE>(smem, nt);
+        size_t smem1 = smem_of<R, MODE>(smem, nt);
         if (one_block_per_sm(smem) && smem1 <= kSmemMax) {
+            smem1 = choose_queue<DIM, R, MODE>(smem1, nt, &a.qcap);
             if constexpr (MODE == 0 && ORD == 3) {
                 if (a.perm) {
                     k_particles<DIM, R, 0, GEO, 3, true, true><<<max_items, nt, smem1, st>>>(a);
@@ -1109,6 +1201,7 @@ static cudaError_t launch_t(cudaStream_t st, int max_items, size_t smem, const P
             return cudaGetLastError();
         }
     }
+    smem = choose_queue<DIM, R, MODE>(smem, kThreads, &a.qcap);
     if constexpr (MODE == 0 && ORD == 3) {
         if (a.perm) {   // right after a sort: the kernel that reads through the permutation
             k_particles<DIM, R, 0, GEO, 3, true><<<max_items, kThreads, smem, st>>>(a);
@@ -1123,13 +1216,17 @@ static cudaError_t launch_t(cudaStream_t st, int max_items, size_t smem, const P
 template <int DIM, typename R, int MODE, class GEO, int ORD = 3, bool PERM = false>
 static cudaError_t set_limit_one(int bytes)
 {
+    int qcap;
     cudaError_t e = cudaFuncSetAttribute(k_particles<DIM, R, MODE, GEO, ORD, PERM>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)choose_queue<DIM, R, MODE>((size_t)bytes, kThreads, &qcap));
     if constexpr (GEO::dyn && DIM == 3) {
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(
                 k_particles<DIM, R, MODE, GEO, ORD, PERM, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                (int)std::min(kSmemMax, smem_of<R, MODE>((size_t)bytes, block_threads<R, true>())));
+                (int)std::min(kSmemMax,
+                              choose_queue<DIM, R, MODE>(smem_of<R, MODE>((size_t)bytes, block_threads<R, true>()),
+                                                         block_threads<R, true>(), &qcap)));
     }
     return e;
 }
@@ -1147,6 +1244,7 @@ template <int DIM, typename R, class GEO = GeoDyn>
 static cudaError_t persistent_t(cudaStream_t st, size_t smem, int nruns, const long long *run_cell_base,
                                 PartArgs<R> a, int *grid_blocks, int launch, long long *ant_n, int antennas)
 {
+    smem = choose_queue<DIM, R, 0>(smem, kThreads, &a.qcap);
     constexpr bool both = GEO::dyn && DIM == 3;
     auto fn0 = k_step_persistent<DIM, R, GEO, false>;
     auto fn1 = k_step_persistent<DIM, R, GEO, true>;
@@ -1187,6 +1285,7 @@ inline PartArgs<R> make_args(WorkItem *items, const int *n_items, const RunDev *
 {
     PartArgs<R> a;
     a.far_list = far_list;
+    a.qcap = kQueueCap;
     a.items = items;
     a.n_items = n_items;
     a.runs = runs;
