@@ -314,7 +314,7 @@ int size_particle_buffers(pic_grid *g, long long total)
         dfree(g->old_off[c]);
         g->old_off[c] = nullptr;
     }
-    const long long nchunks = (total + 4095) / 4096;
+    const long long nchunks = (total + sort_chunk(total) - 1) / sort_chunk(total);
     const long long hist = 256 * std::max(1LL, nchunks);
     const long long sums = std::max<long long>((hist + 2047) / 2048, (g->total_tiles + 2047) / 2048) + 1;
     for (int b = 0; b < 2; ++b) {

@@ -109,6 +109,16 @@ struct SortScratch {
     long long sums_capacity = 0;
 };
 
+// Keys per chunk of the radix passes (a block each; the histogram has 256 counts
+// per chunk).  Up to 2^22 particles in short chunks, since a re-sort's movers fill
+// few: at 2^20 particles 6 of 4096 keys, each block alone for 16 rounds of two
+// barriers (256x256 cells, 40 steps: 2.38 -> 2.34 ms; 64^3 of 2 + 2, 20 steps: 3.85 ->
+// 3.81; above, the histogram would take more memory than it is worth).  Not below
+// 2^14, whose histogram of long chunks is scanned in one launch (8192 particles, 50
+// steps: 2.19 ms, 2.22 in short chunks).
+constexpr int kSmallChunk = 512;
+inline int sort_chunk(long long total) { return total > (1LL << 14) && total <= (1LL << 22) ? kSmallChunk : 4096; }
+
 cudaError_t sort_and_build_items(int prec, int dims, cudaStream_t st, long long total, const PoolBuf &src,
                                  const PoolBuf &dst, const GroupDev *groups, const long long *group_base_dev,
                                  int ngroups, const RunDev *runs, int total_tiles, SortScratch &scr,

@@ -19,6 +19,8 @@ namespace pic {
 constexpr int kSortThreads = 256;
 constexpr int kSortItems = 16;
 constexpr int kChunk = kSortThreads * kSortItems;   // keys per chunk
+// the shorter chunks of sort_chunk (pic_internal.h)
+constexpr int kSmallItems = kSmallChunk / kSortThreads;
 constexpr int kScanItems = 8;
 constexpr int kScanSeg = kSortThreads * kScanItems; // elements per scan block
 constexpr int kItemsThreads = 1024;     // threads of the one-block kernels over tiles
@@ -195,14 +197,15 @@ __global__ void k_keys(long long total, const int *cell, const long long *group_
     vals[p] = (unsigned)p;
 }
 
+template <int ITEMS>
 __device__ __forceinline__ void upsweep(const unsigned *keys, long long n, int shift, unsigned *hist, long long nchunks)
 {
     __shared__ unsigned h[256];
     h[threadIdx.x] = 0;
     __syncthreads();
-    const long long base = blockIdx.x * (long long)kChunk;
+    const long long base = blockIdx.x * (long long)(kSortThreads * ITEMS);
 #pragma unroll 4
-    for (int r = 0; r < kSortItems; ++r) {
+    for (int r = 0; r < ITEMS; ++r) {
         const long long idx = base + r * kSortThreads + threadIdx.x;
         if (idx < n) atomicAdd(&h[(keys[idx] >> shift) & 255u], 1u);
     }
@@ -210,28 +213,31 @@ __device__ __forceinline__ void upsweep(const unsigned *keys, long long n, int s
     hist[threadIdx.x * nchunks + blockIdx.x] = h[threadIdx.x];
 }
 
+template <int ITEMS>
 __global__ void k_upsweep(const unsigned *keys, long long n, int shift, unsigned *hist, long long nchunks)
 {
-    upsweep(keys, n, shift, hist, nchunks);
+    upsweep<ITEMS>(keys, n, shift, hist, nchunks);
 }
 
 // The same over a key count held on the device, at most cap (the keys buffers'
 // length): only its chunks take part, and the histogram is laid out for them
 // (hist_n = 256 x their number, written by k_hist_count).
-__global__ void k_hist_count(const unsigned *n_dev, long long cap, unsigned *hist_n)
+__global__ void k_hist_count(const unsigned *n_dev, long long cap, int chunk, unsigned *hist_n)
 {
     const long long n = min((long long)*n_dev, cap);
-    *hist_n = (unsigned)(256 * ((n + kChunk - 1) / kChunk));
+    *hist_n = (unsigned)(256 * ((n + chunk - 1) / chunk));
 }
 
+template <int ITEMS>
 __global__ void k_upsweep_dev(const unsigned *keys, const unsigned *n_dev, long long cap, int shift, unsigned *hist,
                               const unsigned *hist_n)
 {
     const long long nch = *hist_n / 256;
     if (blockIdx.x >= nch) return;
-    upsweep(keys, min((long long)*n_dev, cap), shift, hist, nch);
+    upsweep<ITEMS>(keys, min((long long)*n_dev, cap), shift, hist, nch);
 }
 
+template <int ITEMS>
 __device__ __forceinline__ void downsweep(const unsigned *keys, const unsigned *vals, long long n, int shift,
                                           const unsigned *hist, long long nchunks, unsigned *keys_out,
                                           unsigned *vals_out)
@@ -246,9 +252,9 @@ __device__ __forceinline__ void downsweep(const unsigned *keys, const unsigned *
 #pragma unroll
     for (int w = 0; w < kSortThreads / 32; ++w) wh[w][tid] = 0;
     __syncthreads();
-    const long long base = blockIdx.x * (long long)kChunk;
+    const long long base = blockIdx.x * (long long)(kSortThreads * ITEMS);
     const unsigned lt = (1u << lane) - 1u;
-    for (int r = 0; r < kSortItems; ++r) {
+    for (int r = 0; r < ITEMS; ++r) {
         const long long idx = base + r * kSortThreads + tid;
         const bool valid = idx < n;
         const unsigned key = valid ? keys[idx] : 0u;
@@ -278,13 +284,15 @@ __device__ __forceinline__ void downsweep(const unsigned *keys, const unsigned *
     }
 }
 
+template <int ITEMS>
 __global__ void __launch_bounds__(kSortThreads) k_downsweep(const unsigned *keys, const unsigned *vals, long long n,
                                                             int shift, const unsigned *hist, long long nchunks,
                                                             unsigned *keys_out, unsigned *vals_out)
 {
-    downsweep(keys, vals, n, shift, hist, nchunks, keys_out, vals_out);
+    downsweep<ITEMS>(keys, vals, n, shift, hist, nchunks, keys_out, vals_out);
 }
 
+template <int ITEMS>
 __global__ void __launch_bounds__(kSortThreads) k_downsweep_dev(const unsigned *keys, const unsigned *vals,
                                                                 const unsigned *n_dev, long long cap, int shift,
                                                                 const unsigned *hist, const unsigned *hist_n,
@@ -292,7 +300,7 @@ __global__ void __launch_bounds__(kSortThreads) k_downsweep_dev(const unsigned *
 {
     const long long nch = *hist_n / 256;
     if (blockIdx.x >= nch) return;
-    downsweep(keys, vals, min((long long)*n_dev, cap), shift, hist, nch, keys_out, vals_out);
+    downsweep<ITEMS>(keys, vals, min((long long)*n_dev, cap), shift, hist, nch, keys_out, vals_out);
 }
 
 // Bank interleave inside every tile.  The particle kernels stage the tile's
@@ -1253,7 +1261,9 @@ cudaError_t sort_and_build_items(int prec, int dims, cudaStream_t st, long long 
     const unsigned nbp = (unsigned)((total + nt - 1) / nt);
     int nbits = 1;
     while ((1ll << nbits) < (long long)total_tiles) ++nbits;
-    const long long nchunks = (total + kChunk - 1) / kChunk;
+    const int chunk = sort_chunk(total);
+    const bool small = chunk == kSmallChunk;
+    const long long nchunks = (total + chunk - 1) / chunk;
     int cur = 0;
     if (resort && !lane_cell) {
         // tile_start holds the previous sort's segments of this pool
@@ -1283,19 +1293,19 @@ cudaError_t sort_and_build_items(int prec, int dims, cudaStream_t st, long long 
         *launches += 1;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         unsigned *hist_n = scr.m_total + 1;
-        k_hist_count<<<1, 1, 0, st>>>(scr.m_total, total, hist_n);
+        k_hist_count<<<1, 1, 0, st>>>(scr.m_total, total, chunk, hist_n);
         *launches += 1;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         for (int shift = 0; shift < nbits; shift += 8) {
-            k_upsweep_dev<<<(unsigned)nchunks, kSortThreads, 0, st>>>(scr.keys[cur], scr.m_total, total, shift,
-                                                                      scr.hist, hist_n);
+            const auto up = small ? k_upsweep_dev<kSmallItems> : k_upsweep_dev<kSortItems>;
+            const auto down = small ? k_downsweep_dev<kSmallItems> : k_downsweep_dev<kSortItems>;
+            up<<<(unsigned)nchunks, kSortThreads, 0, st>>>(scr.keys[cur], scr.m_total, total, shift, scr.hist, hist_n);
             *launches += 1;
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
             if ((e = exclusive_scan_dev(scr.hist, 256 * nchunks, hist_n, scr.block_sums, st, launches)) != cudaSuccess)
                 return e;
-            k_downsweep_dev<<<(unsigned)nchunks, kSortThreads, 0, st>>>(scr.keys[cur], scr.vals[cur], scr.m_total,
-                                                                        total, shift, scr.hist, hist_n,
-                                                                        scr.keys[1 - cur], scr.vals[1 - cur]);
+            down<<<(unsigned)nchunks, kSortThreads, 0, st>>>(scr.keys[cur], scr.vals[cur], scr.m_total, total, shift,
+                                                             scr.hist, hist_n, scr.keys[1 - cur], scr.vals[1 - cur]);
             *launches += 1;
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
             cur = 1 - cur;
@@ -1347,13 +1357,14 @@ cudaError_t sort_and_build_items(int prec, int dims, cudaStream_t st, long long 
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
 
     for (int shift = 0; shift < nbits; shift += 8) {
-        k_upsweep<<<(unsigned)nchunks, kSortThreads, 0, st>>>(scr.keys[cur], total, shift, scr.hist, nchunks);
+        const auto up = small ? k_upsweep<kSmallItems> : k_upsweep<kSortItems>;
+        const auto down = small ? k_downsweep<kSmallItems> : k_downsweep<kSortItems>;
+        up<<<(unsigned)nchunks, kSortThreads, 0, st>>>(scr.keys[cur], total, shift, scr.hist, nchunks);
         *launches += 1;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         if ((e = exclusive_scan(scr.hist, 256 * nchunks, scr.block_sums, st, launches)) != cudaSuccess) return e;
-        k_downsweep<<<(unsigned)nchunks, kSortThreads, 0, st>>>(scr.keys[cur], scr.vals[cur], total, shift,
-                                                                scr.hist, nchunks, scr.keys[1 - cur],
-                                                                scr.vals[1 - cur]);
+        down<<<(unsigned)nchunks, kSortThreads, 0, st>>>(scr.keys[cur], scr.vals[cur], total, shift, scr.hist, nchunks,
+                                                         scr.keys[1 - cur], scr.vals[1 - cur]);
         *launches += 1;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         cur = 1 - cur;
@@ -1453,10 +1464,10 @@ cudaError_t radix_sort_pairs(cudaStream_t st, long long n, int nbits, unsigned *
     const long long nchunks = (n + kChunk - 1) / kChunk;
     int cur = 0;
     for (int shift = 0; shift < nbits; shift += 8) {
-        k_upsweep<<<(unsigned)nchunks, kSortThreads, 0, st>>>(keys[cur], n, shift, hist, nchunks);
+        k_upsweep<kSortItems><<<(unsigned)nchunks, kSortThreads, 0, st>>>(keys[cur], n, shift, hist, nchunks);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         if ((e = exclusive_scan(hist, 256 * nchunks, block_sums, st, &launches)) != cudaSuccess) return e;
-        k_downsweep<<<(unsigned)nchunks, kSortThreads, 0, st>>>(keys[cur], vals[cur], n, shift, hist, nchunks,
+        k_downsweep<kSortItems><<<(unsigned)nchunks, kSortThreads, 0, st>>>(keys[cur], vals[cur], n, shift, hist, nchunks,
                                                                 keys[1 - cur], vals[1 - cur]);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         cur = 1 - cur;
