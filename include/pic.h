@@ -227,8 +227,9 @@ int pic_set_antenna(pic_grid *g, int run, const pic_antenna_desc *a);
 /* Sort policy of pic_step.  By default particles are re-sorted by tile every
  * sort_interval steps.  With adaptive != 0, pic_step times every step's
  * particle kernel and counts the particles that ran more than `halo` cells
- * past their tile since the last sort (they take the slower global-memory
- * path).  While there are such particles it sums the kernel's time above that
+ * past their staged tile (they take the slower global-memory path; a work item
+ * with many such particles stages its tile moved with them).  While there are
+ * such particles it sums the kernel's time above that
  * of the first step after the last sort, and sorts before the next step once
  * the sum, plus the last step's excess again (the next step costs at least as
  * much), exceeds the measured time of a sort.  A sort so triggered after k
@@ -319,9 +320,9 @@ int pic_step_graph(pic_grid *g, int nsteps);
  * synchronizes the stream and returns, per group, the summed device time in
  * milliseconds and the number of groups timed since the last pic_profile(g, 1). */
 enum {
-    PIC_PROF_YEE_B = 0,       /* B half steps (with the J clear) */
+    PIC_PROF_YEE_B = 0,       /* B half steps of their own (the first of a step with the J clear) */
     PIC_PROF_PARTICLES = 1,   /* the particle kernel(s): fused step, gather_push or deposit */
-    PIC_PROF_YEE_E = 2,       /* E full step */
+    PIC_PROF_YEE_E = 2,       /* E full step, with the second B half step where pic_step takes both in one pass */
     PIC_PROF_SORT = 3,        /* the tile sort and work-list build */
     PIC_PROF_N = 4
 };
