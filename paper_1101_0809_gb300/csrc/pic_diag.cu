@@ -189,10 +189,10 @@ struct GlobalZeroB5 {   // offsets -2..2 from the l_a = 2 1/2 base index
 // ORD = 5 (l_a = 2 1/2): E and rho tiles with a halo of (halo + 2) cells, the
 // 4-cell cubic weights around the base index.  ORD = 4 (Eq. wrong1): the same
 // halo for its gather, the l_a = 1 1/2 charge.
-// Three blocks per SM, at the price of spills (96^3 cells of 8 + 8 particles: a step
-// pass with diagnostics 5.69 ms, 5.79 at two blocks without spills).
+// Four blocks per SM, at the price of spills (96^3 cells of 8 + 8 particles: a step
+// pass with diagnostics 5.48 ms, 5.52 at three blocks, about 5.6 at two without spills).
 template <int DIM, int ORD = 3>
-__global__ void __launch_bounds__(kDiagThreads, 3) k_diag_items(int run, const WorkItem *items, const int *n_items,
+__global__ void __launch_bounds__(kDiagThreads, 4) k_diag_items(int run, const WorkItem *items, const int *n_items,
                                                              const GroupDev *groups, const RunDev *runs, Pool<float> P,
                                                              Fields<float> F, int halo, double *rho, double *partials)
 {

@@ -138,10 +138,10 @@ __device__ __forceinline__ int local_coord(int i, int o, int T, int G, int n)
 // tile's particles along together: for a slab behind a wave of a0 = 5, 4x4x4
 // tiles, halo 2 and a sort every 10 steps, the tenth step took 8.0 ms with the
 // tile staged where it was sorted (the first 0.8 ms).  One cell per thread is
-// read, and only by items that had an eighth of their particles (summed over the
-// steps since the sort) on the global-memory path: for the few that leave a tile
-// of a thermal plasma, which has no common drift to follow, the read cost more
-// than it gave (8x8x8 tiles, 20 steps: 8.07 -> 8.9 ms when one was enough).
+// read, and only by items that had one in 256 of their particles (summed over
+// the steps since the sort) on the global-memory path: the slab's ten steps take
+// 16.6 ms with one in 8, 14.9 with one in 64, 14.6 with one in 256; a thermal
+// plasma's few (8x8x8 tiles, sort every 10 steps) cost the same 6.33 ms with each.
 template <int DIM, typename R, bool OLD, int NT>
 __device__ __forceinline__ void item_shift(const PartArgs<R> &a, const WorkItem &it, const RunDev &rn, const int T[3],
                                            int o[3])
@@ -356,7 +356,7 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
     const int ty = (it.tile / rn.ntile[0]) % rn.ntile[1];
     const int tz = DIM == 3 ? it.tile / (rn.ntile[0] * rn.ntile[1]) : 0;
     int org[3] = {tx * T0, ty * T1, tz * T2};
-    if (!RP && 8LL * it.drifted > it.end - it.begin) {   // uniform over the block; none right after a sort
+    if (!RP && 256LL * it.drifted > it.end - it.begin) {   // uniform over the block; none right after a sort
         const int T[3] = {T0, T1, T2};
         item_shift<DIM, R, MODE == 2, NT>(a, it, rn, T, org);
     }
