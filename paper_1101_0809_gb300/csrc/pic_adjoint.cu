@@ -883,15 +883,12 @@ static cudaError_t adj_part_t(cudaStream_t st, const AdjLaunch &lc, const PoolBu
     a.lam_cur = lc.lam_cur;
     if (lc.total <= 0) return cudaSuccess;
     if (lc.items && lc.max_items > 0) {
-        // blocks per work item: as many as give every SM two, of about 512 particles
-        // or more on average.  A block's tiles (18 staged or cleared, 12 flushed)
-        // cost more than its share of the particles gains once the chip is full: 256
-        // items of 4096 particles, 40 steps of the differentiable run: 13.5 ms in
-        // five blocks per item, 13.25 in two, 13.0 in one.
-        int dev = 0, sms = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        const long long ns = std::min(lc.total / ((long long)lc.max_items * 512), 2LL * sms / lc.max_items);
+        // blocks per work item: one for every 512 particles of an average item.  One
+        // block per item stages and flushes fewer tiles, which helps when ids follow
+        // the cells (256 items of 4096 particles: 0.129 ms an adjoint step against
+        // 0.139), but with ids in random order the particles' scattered reads and
+        // writes want more warps: 0.200 ms against 0.158.
+        const long long ns = lc.total / ((long long)lc.max_items * 512);
         const int nsplit = (int)(ns < 1 ? 1 : ns > 8 ? 8 : ns);
         const size_t smem = adjoint_smem_bytes(DIM, sizeof(R) == 8 ? 0 : 1, lc.tile, lc.halo, lc.pitch);
         k_particles_adj_tiled<DIM, R><<<(unsigned)((long long)lc.max_items * nsplit), kThreads, smem, st>>>(
