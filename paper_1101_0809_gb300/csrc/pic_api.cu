@@ -529,6 +529,9 @@ int launch_fields(pic_grid *g, int which, int zero_j)
     return PIC_OK;
 }
 
+// Bytes from one field array to the next in an allocation of several.
+size_t field_part(const pic_grid *g) { return (g->total_cells * elem(g) + 255) & ~(size_t)255; }
+
 // The optional second field buffers: one allocation, given up for particles when
 // memory runs out.  Not an allocation that pic_inject_alloc_failure counts, since
 // none of the calls fails without it.
@@ -565,7 +568,7 @@ cudaError_t drop_second_fields(pic_grid *g, bool keep)
 
 void make_second_fields(pic_grid *g)
 {
-    const size_t part = (g->total_cells * elem(g) + 255) & ~(size_t)255;
+    const size_t part = field_part(g);
     if (cudaMalloc(&g->EB1, 6 * part) != cudaSuccess) {
         cudaGetLastError();
         g->EB1 = nullptr;
@@ -757,10 +760,8 @@ void destroy_grid(pic_grid *g)
     if (!g) return;
     cudaStreamSynchronize(g->stream);   // work still in flight may use the buffers freed below
     drop_second_fields(g, false);
+    dfree(g->EBJ);
     for (int c = 0; c < 3; ++c) {
-        dfree(g->E[c]);
-        dfree(g->B[c]);
-        dfree(g->J[c]);
         dfree(g->old_off[c]);
     }
     dfree(g->old_cell);
@@ -845,14 +846,13 @@ int pic_create_batch(const pic_grid_desc *descs, int nruns, pic_grid **out)
         return r;
     };
     cudaError_t e;
+    if ((e = dalloc_bytes(&g->EBJ, 9 * field_part(g))) != cudaSuccess) return bail(e, "fields");
     for (int c = 0; c < 3; ++c) {
-        if ((e = dalloc_bytes(&g->E[c], g->total_cells * elem(g))) != cudaSuccess) return bail(e, "E");
-        if ((e = dalloc_bytes(&g->B[c], g->total_cells * elem(g))) != cudaSuccess) return bail(e, "B");
-        if ((e = dalloc_bytes(&g->J[c], g->total_cells * elem(g))) != cudaSuccess) return bail(e, "J");
-        if ((e = cudaMemsetAsync(g->E[c], 0, g->total_cells * elem(g), g->stream)) != cudaSuccess) return bail(e, "E");
-        if ((e = cudaMemsetAsync(g->B[c], 0, g->total_cells * elem(g), g->stream)) != cudaSuccess) return bail(e, "B");
-        if ((e = cudaMemsetAsync(g->J[c], 0, g->total_cells * elem(g), g->stream)) != cudaSuccess) return bail(e, "J");
+        g->E[c] = static_cast<char *>(g->EBJ) + c * field_part(g);
+        g->B[c] = static_cast<char *>(g->EBJ) + (3 + c) * field_part(g);
+        g->J[c] = static_cast<char *>(g->EBJ) + (6 + c) * field_part(g);
     }
+    if ((e = cudaMemsetAsync(g->EBJ, 0, 9 * field_part(g), g->stream)) != cudaSuccess) return bail(e, "fields");
     std::vector<RunDev> rds;
     for (auto &r : g->runs) rds.push_back(r.dev);
     if ((e = dalloc(&g->d_runs, rds.size())) != cudaSuccess) return bail(e, "runs");
@@ -1092,6 +1092,8 @@ static int load_many(pic_grid *g, std::vector<LoadReq> &reqs, int on_device)
             if (&o != &q && o.run == q.run && o.species == q.species)
                 return fail(PIC_ERR_INVALID_ARG, "species %d of run %d appears twice", q.species, q.run);
     }
+    const int rs = settle(g);   // a sort left pending would be applied over the loaded records
+    if (rs != PIC_OK) return rs;
     CK(cudaStreamSynchronize(g->stream), "load: prior work");
     // device pointers of every request's x and w (staged if on the host)
     std::vector<std::array<const double *, 6>> src(reqs.size());

@@ -240,6 +240,7 @@ struct pic_grid {
     void *E[3] = {nullptr, nullptr, nullptr};
     void *B[3] = {nullptr, nullptr, nullptr};
     void *J[3] = {nullptr, nullptr, nullptr};
+    void *EBJ = nullptr;            // their one allocation
     // the buffers that the pass of the second B half step and the E step writes, swapped
     // with E and B then; null when there was no memory for them (the step then
     // takes two passes in place)
