@@ -544,26 +544,23 @@ void swap_fields(pic_grid *g)
     g->in_EB1 = !g->in_EB1;
 }
 
-// Frees them, with E and B back in their first buffers.
-cudaError_t drop_second_fields(pic_grid *g, bool keep)
+// E and B back in their first buffers after a step that failed between two passes.
+void fields_home(pic_grid *g)
 {
-    if (!g->EB1) return cudaSuccess;
-    cudaError_t e = cudaSuccess;
-    if (g->in_EB1) {
-        for (int c = 0; c < 3 && keep && e == cudaSuccess; ++c) {
-            const size_t b = g->total_cells * elem(g);
-            e = cudaMemcpyAsync(g->E1[c], g->E[c], b, cudaMemcpyDeviceToDevice, g->stream);
-            if (e == cudaSuccess) e = cudaMemcpyAsync(g->B1[c], g->B[c], b, cudaMemcpyDeviceToDevice, g->stream);
-        }
-        if (e == cudaSuccess && keep) e = cudaStreamSynchronize(g->stream);
-        if (e != cudaSuccess) return e;
-        swap_fields(g);
-        graph_drop(g);
+    if (!g->in_EB1) return;
+    const size_t b = g->total_cells * elem(g);
+    for (int c = 0; c < 3; ++c) {
+        cudaMemcpyAsync(g->E1[c], g->E[c], b, cudaMemcpyDeviceToDevice, g->stream);
+        cudaMemcpyAsync(g->B1[c], g->B[c], b, cudaMemcpyDeviceToDevice, g->stream);
     }
+    swap_fields(g);
+}
+
+void drop_second_fields(pic_grid *g)
+{
     dfree(g->EB1);
     g->EB1 = nullptr;
     for (int c = 0; c < 3; ++c) g->E1[c] = g->B1[c] = nullptr;
-    return e;
 }
 
 void make_second_fields(pic_grid *g)
@@ -580,8 +577,7 @@ void make_second_fields(pic_grid *g)
     }
 }
 
-// Whether the stream is being captured by the caller: a graph of its own must not
-// leave the step's fields in other buffers than it found them in.
+// Whether the stream is being captured by the caller.
 bool stream_captured(const pic_grid *g)
 {
     cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
@@ -590,13 +586,13 @@ bool stream_captured(const pic_grid *g)
 }
 
 // The end of a step, after the deposit: B half step and E step, in one pass into
-// the second buffers unless there are none or `in_place`.  With the few-tile sort
+// the other buffers unless `in_place`.  With the few-tile sort
 // kernels (k_items_one), 40 steps of 256x256 cells FP32: 2.66 -> 2.42 ms, 50 of
 // 32x32 FP64: 2.48 -> 2.28 ms.
 int launch_fields_end(pic_grid *g, bool in_place)
 {
     int rc;
-    if (!g->EB1 || in_place) {
+    if (in_place) {
         if ((rc = launch_fields(g, PIC_B_HALF, 0)) != PIC_OK) return rc;
         return launch_fields(g, PIC_E_FULL, 0);
     }
@@ -609,7 +605,6 @@ int launch_fields_end(pic_grid *g, bool in_place)
         launch_count_add(g, 1);
         if (e != cudaSuccess) return cuda_fail(e, "vector potential");
     }
-    graph_drop(g);   // a captured graph assumes the buffers that E and B were in
     e = launch_yee_b_half_e(g->dims, g->prec, g->stream, g->d_runs, (int)g->runs.size(), maxc, g->E, g->B, g->J,
                             g->E1, g->B1, g->d_ant_n);
     launch_count_add(g, 1);
@@ -759,7 +754,7 @@ void destroy_grid(pic_grid *g)
 {
     if (!g) return;
     cudaStreamSynchronize(g->stream);   // work still in flight may use the buffers freed below
-    drop_second_fields(g, false);
+    drop_second_fields(g);
     dfree(g->EBJ);
     for (int c = 0; c < 3; ++c) {
         dfree(g->old_off[c]);
@@ -1211,8 +1206,8 @@ static int load_many(pic_grid *g, std::vector<LoadReq> &reqs, int on_device)
         cudaGetLastError();
         free_pool(np);
         free_pool(na);
-        e = drop_second_fields(g, true);
-        if (e == cudaSuccess) e = alloc_pool(g, np, total);
+        drop_second_fields(g);
+        e = alloc_pool(g, np, total);
         if (e == cudaSuccess) e = alloc_pool(g, na, total);
     }
     if (e != cudaSuccess) {
@@ -1377,17 +1372,23 @@ int pic_sort(pic_grid *g)
     return do_sort(g);
 }
 
-int pic_step(pic_grid *g, int nsteps)
+static int save_body(pic_grid *g, void *dst, int on_device);
+
+// nsteps steps; with states, a device snapshot before each of them.  E and B
+// change buffers in pairs of steps only: a call finds and leaves them where they
+// were created, so that a graph that the caller captured from this or another
+// call stays valid.  A last step without a partner, and every step that the
+// caller captures, takes the two passes in place.
+static int run_steps(pic_grid *g, int nsteps, void *const *states)
 {
-    if (!g) return fail(PIC_ERR_INVALID_ARG, "null grid");
-    if (nsteps < 0) return fail(PIC_ERR_INVALID_ARG, "negative step count");
     const bool measure = g->adaptive_sort && g->total > 0;
-    const bool in_place = stream_captured(g);
+    const bool pairs = g->EB1 && !stream_captured(g);
     if (measure && !g->ad_ev[0])
         for (auto &ev : g->ad_ev) CK(cudaEventCreate(&ev), "sort policy events");
     for (int s = 0; s < nsteps; ++s) {
         int rc;
         bool timed_sort = false;
+        if (states && (rc = save_body(g, states[s], 1)) != PIC_OK) return rc;
         const int limit = measure && g->ad_limit > 0 ? std::min(g->ad_limit, g->sort_interval) : g->sort_interval;
         if (measure && g->steps_since_sort >= limit && !g->sort_due && g->steps_since_sort > 0) {
             // a cycle that reached the learned interval without drift: after
@@ -1417,7 +1418,8 @@ int pic_step(pic_grid *g, int nsteps)
         if (measure) CK(cudaEventRecord(g->ad_ev[0], g->stream), "sort policy events");
         if (g->total > 0 && (rc = launch_part(g, 0)) != PIC_OK) return rc;
         if (measure) CK(cudaEventRecord(g->ad_ev[1], g->stream), "sort policy events");
-        if ((rc = launch_fields_end(g, in_place)) != PIC_OK) return rc;
+        const bool pair = pairs && (g->in_EB1 || s + 1 < nsteps);
+        if ((rc = launch_fields_end(g, !pair)) != PIC_OK) return rc;
         g->steps_since_sort += 1;
         g->have_old = false;
         if (measure) {
@@ -1456,6 +1458,15 @@ int pic_step(pic_grid *g, int nsteps)
         }
     }
     return PIC_OK;
+}
+
+int pic_step(pic_grid *g, int nsteps)
+{
+    if (!g) return fail(PIC_ERR_INVALID_ARG, "null grid");
+    if (nsteps < 0) return fail(PIC_ERR_INVALID_ARG, "negative step count");
+    const int rc = run_steps(g, nsteps, nullptr);
+    fields_home(g);
+    return rc;
 }
 
 // One step of every run in one cooperative launch (plus the sort launches
@@ -1886,12 +1897,9 @@ int pic_step_saving(pic_grid *g, int nsteps, void *const *states)
     if (nsteps < 0) return fail(PIC_ERR_INVALID_ARG, "negative step count");
     for (int s = 0; s < nsteps; ++s)
         if (!states[s]) return fail(PIC_ERR_INVALID_ARG, "null state buffer %d", s);
-    for (int s = 0; s < nsteps; ++s) {
-        int rc = save_body(g, states[s], 1);
-        if (rc == PIC_OK) rc = pic_step(g, 1);
-        if (rc != PIC_OK) return rc;
-    }
-    return PIC_OK;
+    const int rc = run_steps(g, nsteps, states);
+    fields_home(g);
+    return rc;
 }
 
 // ---- adjoint ---------------------------------------------------------------------

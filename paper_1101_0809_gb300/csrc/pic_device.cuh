@@ -1126,6 +1126,10 @@ __device__ __forceinline__ double antenna_field(const RunDev &rn, double x, doub
     return rn.ant_E0 * g * sin(rn.ant_omega * tau);
 }
 
+// v + k f, rounded as the precision's other field sums are.
+__device__ __forceinline__ double add_incident(double v, double k, double f) { return fma(k, f, v); }
+__device__ __forceinline__ float add_incident(float v, double k, double f) { return v + (float)(k * f); }
+
 // The cell indices of cell l of a run (fewer than 2^31 cells).  The 64-bit
 // quotients that stood here set the Yee kernels' time: 256x64x64 cells FP32 took
 // 20.9 us per B half step and 24.0 us per E step, 48 and 60 bytes per cell.
@@ -1135,6 +1139,27 @@ __device__ __forceinline__ void yee_ijk(const RunDev &rn, int l, int &i, int &j,
     i = l - r * rn.n[0];
     k = divu31(r, rn.div_ny);
     j = r - k * rn.n[1];
+}
+
+// The B half step's new values at a cell, h = c dt/(2 d): the fused multiply-adds
+// are written out, so that the two passes and the one pass round alike and a
+// run's fields do not depend on how its steps are split into calls.
+template <int DIM, typename R>
+__device__ __forceinline__ R yee_bx(R b, R hy, R hz, R ez, R ez_j, R ey, R ey_k)
+{
+    b = fma(-hy, ez - ez_j, b);
+    return DIM == 3 ? fma(hz, ey - ey_k, b) : b;
+}
+template <int DIM, typename R>
+__device__ __forceinline__ R yee_by(R b, R hx, R hz, R ez, R ez_i, R ex, R ex_k)
+{
+    b = fma(hx, ez - ez_i, b);
+    return DIM == 3 ? fma(-hz, ex - ex_k, b) : b;
+}
+template <typename R>
+__device__ __forceinline__ R yee_bz(R b, R hx, R hy, R ey, R ey_i, R ex, R ex_j)
+{
+    return fma(hy, ex - ex_j, fma(-hx, ey - ey_i, b));
 }
 
 // ant_n: the antenna clock of the run (E steps since the antenna was set).
@@ -1150,20 +1175,16 @@ __device__ __forceinline__ void yee_b_half_cell(const RunDev &rn, const Fields<R
     const long long pjm = p + (long long)nx * (j == 0 ? ny - 1 : -1);
     const bool f32 = sizeof(R) == 4;
     const R hx = f32 ? R(0.5f * rn.cNf[0]) : R(0.5 * rn.cN[0]), hy = f32 ? R(0.5f * rn.cNf[1]) : R(0.5 * rn.cN[1]);
+    const R hz = f32 ? R(0.5f * rn.cNf[2]) : R(0.5 * rn.cN[2]);
+    const long long pkm = DIM == 3 ? p + (long long)nx * ny * (k == 0 ? nz - 1 : -1) : p;
     const R ex = F.E[0][p], ey = F.E[1][p], ez = F.E[2][p];
-    R bx = F.B[0][p] - hy * (ez - F.E[2][pjm]);
-    R by = F.B[1][p] + hx * (ez - F.E[2][pim]);
-    R bz = F.B[2][p] - hx * (ey - F.E[1][pim]) + hy * (ex - F.E[0][pjm]);
-    if (DIM == 3) {
-        const long long pkm = p + (long long)nx * ny * (k == 0 ? nz - 1 : -1);
-        const R hz = f32 ? R(0.5f * rn.cNf[2]) : R(0.5 * rn.cN[2]);
-        bx += hz * (ey - F.E[1][pkm]);
-        by -= hz * (ex - F.E[0][pkm]);
-    }
+    const R bx = yee_bx<DIM>(F.B[0][p], hy, hz, ez, F.E[2][pjm], ey, DIM == 3 ? F.E[1][pkm] : R(0));
+    R by = yee_by<DIM>(F.B[1][p], hx, hz, ez, F.E[2][pim], ex, DIM == 3 ? F.E[0][pkm] : R(0));
+    R bz = yee_bz(F.B[2][p], hx, hy, ey, F.E[1][pim], ex, F.E[0][pjm]);
     if (rn.ant_pol != 0 && i == rn.ant_i0) {
         // the scattered-field E node at x = i0 - 1/2 lacks the incident wave
-        const R a = R(0.5 * rn.cN[0] * antenna_field(rn, rn.ant_i0 - 0.5, ant_n * rn.dt));
-        if (rn.ant_pol == 1) bz += a; else by -= a;
+        const double h = 0.5 * rn.cN[0], f = antenna_field(rn, rn.ant_i0 - 0.5, ant_n * rn.dt);
+        if (rn.ant_pol == 1) bz = add_incident(bz, h, f); else by = add_incident(by, -h, f);
     }
     F.B[0][p] = bx;
     F.B[1][p] = by;
@@ -1183,19 +1204,19 @@ __device__ __forceinline__ void yee_e_values(const RunDev &rn, const R e0[3], co
     const bool f32 = sizeof(R) == 4;
     const R cx = f32 ? R(rn.cNf[0]) : R(rn.cN[0]), cy = f32 ? R(rn.cNf[1]) : R(rn.cN[1]);
     const R fp = f32 ? R(rn.fpdtf) : R(rn.fpdt);
-    e[0] = e0[0] - fp * J[0] + cy * (bz_j - bz);
-    e[1] = e0[1] - fp * J[1] - cx * (bz_i - bz);
-    e[2] = e0[2] - fp * J[2] + cx * (by_i - by) - cy * (bx_j - bx);
+    e[0] = fma(cy, bz_j - bz, fma(-fp, J[0], e0[0]));
+    e[1] = fma(-cx, bz_i - bz, fma(-fp, J[1], e0[1]));
+    e[2] = fma(-cy, bx_j - bx, fma(cx, by_i - by, fma(-fp, J[2], e0[2])));
     if (DIM == 3) {
         const R cz = f32 ? R(rn.cNf[2]) : R(rn.cN[2]);
-        e[0] -= cz * (by_k - by);
-        e[1] += cz * (bx_k - bx);
+        e[0] = fma(-cz, by_k - by, e[0]);
+        e[1] = fma(cz, bx_k - bx, e[1]);
     }
     if (rn.ant_pol != 0 && i == rn.ant_i0 - 1) {
         // the scattered-field E node at x = i0 - 1/2 sees the total-field B node at
         // x = i0, whose incident part (B_z = E_inc, B_y = -E_inc) comes off
-        const R a = R(rn.cN[0] * antenna_field(rn, rn.ant_i0, (ant_n + 0.5) * rn.dt));
-        if (rn.ant_pol == 1) e[1] += a; else e[2] += a;
+        const double f = antenna_field(rn, rn.ant_i0, (ant_n + 0.5) * rn.dt);
+        if (rn.ant_pol == 1) e[1] = add_incident(e[1], rn.cN[0], f); else e[2] = add_incident(e[2], rn.cN[0], f);
     }
 }
 
@@ -1241,17 +1262,15 @@ __device__ __forceinline__ void yee_b_half_e_cell(const RunDev &rn, const Fields
     const long long kp = DIM == 3 ? nxy * (k == nz - 1 ? -(nz - 1) : 1) : 0;
     // the new B of the cell at q whose neighbours below are at qi, qj, qk
     auto nbx = [&](long long q, long long qj, long long qk) {
-        R b = F.B[0][q] - hy * (F.E[2][q] - F.E[2][qj]);
-        if (DIM == 3) b += hz * (F.E[1][q] - F.E[1][qk]);
-        return b;
+        return yee_bx<DIM>(F.B[0][q], hy, hz, F.E[2][q], F.E[2][qj], DIM == 3 ? F.E[1][q] : R(0),
+                           DIM == 3 ? F.E[1][qk] : R(0));
     };
     auto nby = [&](long long q, long long qi, long long qk) {
-        R b = F.B[1][q] + hx * (F.E[2][q] - F.E[2][qi]);
-        if (DIM == 3) b -= hz * (F.E[0][q] - F.E[0][qk]);
-        return b;
+        return yee_by<DIM>(F.B[1][q], hx, hz, F.E[2][q], F.E[2][qi], DIM == 3 ? F.E[0][q] : R(0),
+                           DIM == 3 ? F.E[0][qk] : R(0));
     };
     auto nbz = [&](long long q, long long qi, long long qj) {
-        return F.B[2][q] - hx * (F.E[1][q] - F.E[1][qi]) + hy * (F.E[0][q] - F.E[0][qj]);
+        return yee_bz(F.B[2][q], hx, hy, F.E[1][q], F.E[1][qi], F.E[0][q], F.E[0][qj]);
     };
     R bx = nbx(p, p + jm, p + km), by = nby(p, p + im, p + km), bz = nbz(p, p + im, p + jm);
     R bx_j = nbx(p + jp, p, p + jp + km), bz_j = nbz(p + jp, p + jp + im, p);
@@ -1264,12 +1283,13 @@ __device__ __forceinline__ void yee_b_half_e_cell(const RunDev &rn, const Fields
     if (rn.ant_pol != 0 && (i == rn.ant_i0 || i + 1 == rn.ant_i0)) {
         // the scattered-field E node at x = i0 - 1/2 lacks the incident wave
         // (1 <= i0 < nx, so the + neighbour along x at i0 is not across the wrap)
-        const R a = R(0.5 * rn.cN[0] * antenna_field(rn, rn.ant_i0 - 0.5, ant_n * rn.dt));
+        const double h = 0.5 * rn.cN[0], f = antenna_field(rn, rn.ant_i0 - 0.5, ant_n * rn.dt);
         const bool z = rn.ant_pol == 1;
+        auto add = [&](R &v) { v = add_incident(v, z ? h : -h, f); };
         if (i == rn.ant_i0) {
-            if (z) { bz += a; bz_j += a; } else { by -= a; by_k -= a; }
+            if (z) { add(bz); add(bz_j); } else { add(by); add(by_k); }
         } else {
-            if (z) bz_i += a; else by_i -= a;
+            if (z) add(bz_i); else add(by_i);
         }
     }
     const R e0[3] = {F.E[0][p], F.E[1][p], F.E[2][p]}, J[3] = {F.J[0][p], F.J[1][p], F.J[2][p]};

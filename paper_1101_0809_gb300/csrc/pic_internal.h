@@ -242,12 +242,12 @@ struct pic_grid {
     void *J[3] = {nullptr, nullptr, nullptr};
     void *EBJ = nullptr;            // their one allocation
     // the buffers that the pass of the second B half step and the E step writes, swapped
-    // with E and B then; null when there was no memory for them (the step then
-    // takes two passes in place)
+    // with E and B then and again by the next step of the same call; null when there
+    // was no memory for them (the step then takes two passes in place)
     void *E1[3] = {nullptr, nullptr, nullptr};
     void *B1[3] = {nullptr, nullptr, nullptr};
     void *EB1 = nullptr;            // their one allocation
-    bool in_EB1 = false;            // E and B are in it now (an odd number of swaps)
+    bool in_EB1 = false;            // E and B are in it now (only inside a call that steps)
 
     // species / groups
     std::vector<pic::HostGroup> groups;
