@@ -150,14 +150,12 @@ bool injected_alloc_failure()
     return false;
 }
 
-thread_local bool t_injected = false;   // the thread's last allocation was made to fail
-
 template <typename T>
 cudaError_t dalloc(T **p, size_t count)
 {
     *p = nullptr;
     if (count == 0) return cudaSuccess;
-    if ((t_injected = injected_alloc_failure())) return cudaErrorMemoryAllocation;
+    if (injected_alloc_failure()) return cudaErrorMemoryAllocation;
     return cudaMalloc((void **)p, count * sizeof(T));
 }
 
@@ -165,7 +163,7 @@ cudaError_t dalloc_bytes(void **p, size_t bytes)
 {
     *p = nullptr;
     if (bytes == 0) return cudaSuccess;
-    if ((t_injected = injected_alloc_failure())) return cudaErrorMemoryAllocation;
+    if (injected_alloc_failure()) return cudaErrorMemoryAllocation;
     return cudaMalloc(p, bytes);
 }
 
@@ -190,6 +188,7 @@ cudaError_t alloc_pool(pic_grid *g, PoolBuf &P, long long n)
     const size_t bytes = std::max(2 * wi + (g->dims + 3) * wr, (size_t)n * sizeof(LoadRec));
     const cudaError_t e = dalloc_bytes(&P.slab, bytes);
     if (e != cudaSuccess) return e;
+    P.bytes = bytes;
     unsigned char *at = static_cast<unsigned char *>(P.slab);
     auto take = [&](size_t w) {
         unsigned char *p = at;
@@ -532,49 +531,22 @@ int launch_fields(pic_grid *g, int which, int zero_j)
 // Bytes from one field array to the next in an allocation of several.
 size_t field_part(const pic_grid *g) { return (g->total_cells * elem(g) + 255) & ~(size_t)255; }
 
-// The optional second field buffers: one allocation, given up for particles when
-// memory runs out.  Not an allocation that pic_inject_alloc_failure counts, since
-// none of the calls fails without it.
-void swap_fields(pic_grid *g)
+// E and B at `base`: EBJ, where they are outside of a call that steps, or the
+// unused particle pool.
+void fields_at(pic_grid *g, void *base)
 {
     for (int c = 0; c < 3; ++c) {
-        std::swap(g->E[c], g->E1[c]);
-        std::swap(g->B[c], g->B1[c]);
+        g->E[c] = static_cast<char *>(base) + c * field_part(g);
+        g->B[c] = static_cast<char *>(base) + (3 + c) * field_part(g);
     }
-    g->in_EB1 = !g->in_EB1;
 }
 
-// E and B back in their first buffers after a step that failed between two passes.
+// E and B back in EBJ after a step that failed between two passes.
 void fields_home(pic_grid *g)
 {
-    if (!g->in_EB1) return;
-    const size_t b = g->total_cells * elem(g);
-    for (int c = 0; c < 3; ++c) {
-        cudaMemcpyAsync(g->E1[c], g->E[c], b, cudaMemcpyDeviceToDevice, g->stream);
-        cudaMemcpyAsync(g->B1[c], g->B[c], b, cudaMemcpyDeviceToDevice, g->stream);
-    }
-    swap_fields(g);
-}
-
-void drop_second_fields(pic_grid *g)
-{
-    dfree(g->EB1);
-    g->EB1 = nullptr;
-    for (int c = 0; c < 3; ++c) g->E1[c] = g->B1[c] = nullptr;
-}
-
-void make_second_fields(pic_grid *g)
-{
-    const size_t part = field_part(g);
-    if (cudaMalloc(&g->EB1, 6 * part) != cudaSuccess) {
-        cudaGetLastError();
-        g->EB1 = nullptr;
-        return;
-    }
-    for (int c = 0; c < 3; ++c) {
-        g->E1[c] = static_cast<char *>(g->EB1) + c * part;
-        g->B1[c] = static_cast<char *>(g->EB1) + (3 + c) * part;
-    }
+    if (g->E[0] == g->EBJ) return;
+    cudaMemcpyAsync(g->EBJ, g->E[0], 6 * field_part(g), cudaMemcpyDeviceToDevice, g->stream);
+    fields_at(g, g->EBJ);
 }
 
 // Whether the stream is being captured by the caller.
@@ -586,7 +558,7 @@ bool stream_captured(const pic_grid *g)
 }
 
 // The end of a step, after the deposit: B half step and E step, in one pass into
-// the other buffers unless `in_place`.  With the few-tile sort
+// the other of the two places (fields_at) unless `in_place`.  With the few-tile sort
 // kernels (k_items_one), 40 steps of 256x256 cells FP32: 2.66 -> 2.42 ms, 50 of
 // 32x32 FP64: 2.48 -> 2.28 ms.
 int launch_fields_end(pic_grid *g, bool in_place)
@@ -605,11 +577,15 @@ int launch_fields_end(pic_grid *g, bool in_place)
         launch_count_add(g, 1);
         if (e != cudaSuccess) return cuda_fail(e, "vector potential");
     }
-    e = launch_yee_b_half_e(g->dims, g->prec, g->stream, g->d_runs, (int)g->runs.size(), maxc, g->E, g->B, g->J,
-                            g->E1, g->B1, g->d_ant_n);
+    void *const E[3] = {g->E[0], g->E[1], g->E[2]}, *const B[3] = {g->B[0], g->B[1], g->B[2]};
+    fields_at(g, E[0] == g->EBJ ? g->pool_alt.slab : g->EBJ);
+    e = launch_yee_b_half_e(g->dims, g->prec, g->stream, g->d_runs, (int)g->runs.size(), maxc, E, B, g->J, g->E, g->B,
+                            g->d_ant_n);
     launch_count_add(g, 1);
-    if (e != cudaSuccess) return cuda_fail(e, "Yee kernel");
-    swap_fields(g);
+    if (e != cudaSuccess) {
+        fields_at(g, E[0]);
+        return cuda_fail(e, "Yee kernel");
+    }
     if (g->antennas > 0) {   // the E step ends a step of the antenna clock
         e = launch_antenna_tick(g->stream, g->d_ant_n, (int)g->runs.size());
         launch_count_add(g, 1);
@@ -754,7 +730,6 @@ void destroy_grid(pic_grid *g)
 {
     if (!g) return;
     cudaStreamSynchronize(g->stream);   // work still in flight may use the buffers freed below
-    drop_second_fields(g);
     dfree(g->EBJ);
     for (int c = 0; c < 3; ++c) {
         dfree(g->old_off[c]);
@@ -842,11 +817,8 @@ int pic_create_batch(const pic_grid_desc *descs, int nruns, pic_grid **out)
     };
     cudaError_t e;
     if ((e = dalloc_bytes(&g->EBJ, 9 * field_part(g))) != cudaSuccess) return bail(e, "fields");
-    for (int c = 0; c < 3; ++c) {
-        g->E[c] = static_cast<char *>(g->EBJ) + c * field_part(g);
-        g->B[c] = static_cast<char *>(g->EBJ) + (3 + c) * field_part(g);
-        g->J[c] = static_cast<char *>(g->EBJ) + (6 + c) * field_part(g);
-    }
+    fields_at(g, g->EBJ);
+    for (int c = 0; c < 3; ++c) g->J[c] = static_cast<char *>(g->EBJ) + (6 + c) * field_part(g);
     if ((e = cudaMemsetAsync(g->EBJ, 0, 9 * field_part(g), g->stream)) != cudaSuccess) return bail(e, "fields");
     std::vector<RunDev> rds;
     for (auto &r : g->runs) rds.push_back(r.dev);
@@ -897,7 +869,6 @@ int pic_create_batch(const pic_grid_desc *descs, int nruns, pic_grid **out)
         (e = diag_set_smem_limit(g->dims, diag_items_smem_bytes(g->dims, g->tile, g->halo, g->pitch, g->order2),
                                  g->order2)) != cudaSuccess)
         return bail(e, "smem limit");
-    make_second_fields(g);
     if ((e = cudaStreamSynchronize(g->stream)) != cudaSuccess) return bail(e, "create");
     *out = g;
     return PIC_OK;
@@ -1202,14 +1173,6 @@ static int load_many(pic_grid *g, std::vector<LoadReq> &reqs, int on_device)
     PoolBuf np, na;
     cudaError_t e = alloc_pool(g, np, total);
     if (e == cudaSuccess) e = alloc_pool(g, na, total);
-    if (e == cudaErrorMemoryAllocation && !t_injected && g->EB1) {   // particles before the step's second field buffers
-        cudaGetLastError();
-        free_pool(np);
-        free_pool(na);
-        drop_second_fields(g);
-        e = alloc_pool(g, np, total);
-        if (e == cudaSuccess) e = alloc_pool(g, na, total);
-    }
     if (e != cudaSuccess) {
         free_pool(np);
         free_pool(na);
@@ -1375,14 +1338,18 @@ int pic_sort(pic_grid *g)
 static int save_body(pic_grid *g, void *dst, int on_device);
 
 // nsteps steps; with states, a device snapshot before each of them.  E and B
-// change buffers in pairs of steps only: a call finds and leaves them where they
-// were created, so that a graph that the caller captured from this or another
-// call stays valid.  A last step without a partner, and every step that the
-// caller captures, takes the two passes in place.
+// change places in pairs of steps only, between EBJ and the particle pool that
+// is unused from a sort's particle launch to the next sort: a call finds and
+// leaves them in EBJ, so that a graph that the caller captured from this or
+// another call stays valid, and the one pass takes no memory of its own.  In
+// place, by two passes: a step without a partner, before the next sort or at the
+// call's end; every step that the caller captures or the sort policy measures
+// (its sorts are not known a step ahead); grids whose pool is smaller than the
+// fields.
 static int run_steps(pic_grid *g, int nsteps, void *const *states)
 {
     const bool measure = g->adaptive_sort && g->total > 0;
-    const bool pairs = g->EB1 && !stream_captured(g);
+    const bool pairs = !measure && g->pool_alt.bytes >= 6 * field_part(g) && !stream_captured(g);
     if (measure && !g->ad_ev[0])
         for (auto &ev : g->ad_ev) CK(cudaEventCreate(&ev), "sort policy events");
     for (int s = 0; s < nsteps; ++s) {
@@ -1418,7 +1385,7 @@ static int run_steps(pic_grid *g, int nsteps, void *const *states)
         if (measure) CK(cudaEventRecord(g->ad_ev[0], g->stream), "sort policy events");
         if (g->total > 0 && (rc = launch_part(g, 0)) != PIC_OK) return rc;
         if (measure) CK(cudaEventRecord(g->ad_ev[1], g->stream), "sort policy events");
-        const bool pair = pairs && (g->in_EB1 || s + 1 < nsteps);
+        const bool pair = pairs && (g->E[0] != g->EBJ || (s + 1 < nsteps && g->steps_since_sort + 1 < g->sort_interval));
         if ((rc = launch_fields_end(g, !pair)) != PIC_OK) return rc;
         g->steps_since_sort += 1;
         g->have_old = false;

@@ -32,6 +32,7 @@ struct HostGroup {
 // of one allocation.
 struct PoolBuf {
     void *slab = nullptr;   // the allocation: >= sizeof(LoadRec) per particle in FP32
+    size_t bytes = 0;
     int *cell = nullptr;
     void *off[3] = {nullptr, nullptr, nullptr};
     void *w[3] = {nullptr, nullptr, nullptr};
@@ -240,14 +241,7 @@ struct pic_grid {
     void *E[3] = {nullptr, nullptr, nullptr};
     void *B[3] = {nullptr, nullptr, nullptr};
     void *J[3] = {nullptr, nullptr, nullptr};
-    void *EBJ = nullptr;            // their one allocation
-    // the buffers that the pass of the second B half step and the E step writes, swapped
-    // with E and B then and again by the next step of the same call; null when there
-    // was no memory for them (the step then takes two passes in place)
-    void *E1[3] = {nullptr, nullptr, nullptr};
-    void *B1[3] = {nullptr, nullptr, nullptr};
-    void *EB1 = nullptr;            // their one allocation
-    bool in_EB1 = false;            // E and B are in it now (only inside a call that steps)
+    void *EBJ = nullptr;   // their one allocation, which E and B leave only inside a call that steps (run_steps)
 
     // species / groups
     std::vector<pic::HostGroup> groups;
