@@ -917,14 +917,11 @@ size_t adjoint_smem_bytes(int dims, int prec, const int tile[3], int halo, const
 
 cudaError_t adjoint_set_smem_limit(int dims, int prec, size_t bytes)
 {
-    const int b = (int)bytes;
     if (dims == 3)
-        return prec == 0
-                   ? cudaFuncSetAttribute(k_particles_adj_tiled<3, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, b)
-                   : cudaFuncSetAttribute(k_particles_adj_tiled<3, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-    return prec == 0
-               ? cudaFuncSetAttribute(k_particles_adj_tiled<2, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, b)
-               : cudaFuncSetAttribute(k_particles_adj_tiled<2, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+        return prec == 0 ? allow_smem(k_particles_adj_tiled<3, double>, bytes)
+                         : allow_smem(k_particles_adj_tiled<3, float>, bytes);
+    return prec == 0 ? allow_smem(k_particles_adj_tiled<2, double>, bytes)
+                     : allow_smem(k_particles_adj_tiled<2, float>, bytes);
 }
 
 cudaError_t launch_particles_adj(int dims, int prec, cudaStream_t st, const AdjLaunch &lc, const PoolBuf &P,

@@ -595,15 +595,9 @@ size_t diag_items_smem_bytes(int dims, const int tile[3], int halo, const int pi
 
 cudaError_t diag_set_smem_limit(int dims, size_t bytes, int order2)
 {
-    const int b = (int)bytes;
-    if (order2 == 5)
-        return dims == 3 ? cudaFuncSetAttribute(k_diag_items<3, 5>, cudaFuncAttributeMaxDynamicSharedMemorySize, b)
-                         : cudaFuncSetAttribute(k_diag_items<2, 5>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-    if (order2 == 4)
-        return dims == 3 ? cudaFuncSetAttribute(k_diag_items<3, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, b)
-                         : cudaFuncSetAttribute(k_diag_items<2, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-    return dims == 3 ? cudaFuncSetAttribute(k_diag_items<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, b)
-                     : cudaFuncSetAttribute(k_diag_items<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+    if (order2 == 5) return dims == 3 ? allow_smem(k_diag_items<3, 5>, bytes) : allow_smem(k_diag_items<2, 5>, bytes);
+    if (order2 == 4) return dims == 3 ? allow_smem(k_diag_items<3, 4>, bytes) : allow_smem(k_diag_items<2, 4>, bytes);
+    return dims == 3 ? allow_smem(k_diag_items<3>, bytes) : allow_smem(k_diag_items<2>, bytes);
 }
 
 }  // namespace pic

@@ -39,6 +39,22 @@ struct PoolBuf {
     int *id = nullptr;
 };
 
+// Lets a kernel take all the shared memory that a block can have, `bytes` at
+// least.  The limit is one per kernel and process: set to a grid's own size it
+// would be lowered by the next grid with smaller tiles.
+template <typename Kernel>
+inline cudaError_t allow_smem(Kernel kernel, size_t bytes)
+{
+    int dev = 0, most = 0;
+    cudaFuncAttributes at;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&at, kernel);
+    if (e != cudaSuccess) return e;
+    const int all = most - (int)at.sharedSizeBytes;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, all > (int)bytes ? all : (int)bytes);
+}
+
 // Launch helpers implemented in the .cu files.  All enqueue on `st` and return
 // a cudaError_t from the launch.
 cudaError_t launch_particles(int dims, int prec, int mode, cudaStream_t st, WorkItem *items,

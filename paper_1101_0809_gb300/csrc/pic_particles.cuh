@@ -1216,17 +1216,9 @@ static cudaError_t launch_t(cudaStream_t st, int max_items, size_t smem, PartArg
 template <int DIM, typename R, int MODE, class GEO, int ORD = 3, bool PERM = false>
 static cudaError_t set_limit_one(int bytes)
 {
-    int qcap;
-    cudaError_t e = cudaFuncSetAttribute(k_particles<DIM, R, MODE, GEO, ORD, PERM>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)choose_queue<DIM, R, MODE>((size_t)bytes, kThreads, &qcap));
+    cudaError_t e = allow_smem(k_particles<DIM, R, MODE, GEO, ORD, PERM>, (size_t)bytes);
     if constexpr (GEO::dyn && DIM == 3) {
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(
-                k_particles<DIM, R, MODE, GEO, ORD, PERM, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                (int)std::min(kSmemMax,
-                              choose_queue<DIM, R, MODE>(smem_of<R, MODE>((size_t)bytes, block_threads<R, true>()),
-                                                         block_threads<R, true>(), &qcap)));
+        if (e == cudaSuccess) e = allow_smem(k_particles<DIM, R, MODE, GEO, ORD, PERM, true>, (size_t)bytes);
     }
     return e;
 }
@@ -1261,7 +1253,7 @@ static cudaError_t persistent_t(cudaStream_t st, size_t smem, int nruns, const l
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         for (auto f : {fn0, fn1}) {
-            e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            e = allow_smem(f, smem);
             if (e != cudaSuccess) return e;
             int pf = 0;
             e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pf, f, kThreads, smem);

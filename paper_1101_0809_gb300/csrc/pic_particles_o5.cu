@@ -32,8 +32,7 @@ cudaError_t launch_particles_o5(int dims, int prec, int mode, cudaStream_t st, i
 cudaError_t particles_o5_set_smem_limit(int dims, int prec, int mode, size_t bytes)
 {
     if (dims == 3 && prec != 0 && mode == 0) {
-        const cudaError_t e = cudaFuncSetAttribute(k_particles<3, float, 0, Geo5_444, 5>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        const cudaError_t e = allow_smem(k_particles<3, float, 0, Geo5_444, 5>, bytes);
         if (e != cudaSuccess) return e;
     }
     return particles_ord_set_smem_limit_t<5>(dims, prec, mode, bytes);
