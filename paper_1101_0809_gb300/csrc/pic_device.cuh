@@ -34,7 +34,7 @@ inline DivU31 make_divu31(int d)
     v.L = L;
     return v;
 }
-__device__ __forceinline__ int divu31(int n, const DivU31 &v)
+__host__ __device__ __forceinline__ int divu31(int n, const DivU31 &v)
 {
     return (int)(((unsigned long long)(unsigned)n * v.m) >> v.L);
 }
@@ -1130,13 +1130,21 @@ __device__ __forceinline__ double antenna_field(const RunDev &rn, double x, doub
 __device__ __forceinline__ double add_incident(double v, double k, double f) { return fma(k, f, v); }
 __device__ __forceinline__ float add_incident(float v, double k, double f) { return v + (float)(k * f); }
 
-// The cell indices of cell l of a run (fewer than 2^31 cells).  The 64-bit
-// quotients that stood here set the Yee kernels' time: 256x64x64 cells FP32 took
-// 20.9 us per B half step and 24.0 us per E step, 48 and 60 bytes per cell.
-__device__ __forceinline__ void yee_ijk(const RunDev &rn, int l, int &i, int &j, int &k)
+// The cell indices of cell l of a run.  Without 64-bit quotients below 2^31, where
+// they set the Yee kernels' time (256x64x64 cells FP32: 20.9 us per B half step and
+// 24.0 us per E step, 48 and 60 bytes per cell); a run without particles may
+// have more cells.
+__host__ __device__ __forceinline__ void yee_ijk(const RunDev &rn, long long l, int &i, int &j, int &k)
 {
-    const int r = divu31(l, rn.div_nx);
-    i = l - r * rn.n[0];
+    if (l >> 31 != 0) {
+        const long long r = l / rn.n[0];
+        i = (int)(l - r * rn.n[0]);
+        k = (int)(r / rn.n[1]);
+        j = (int)(r - (long long)k * rn.n[1]);
+        return;
+    }
+    const int r = divu31((int)l, rn.div_nx);
+    i = (int)l - r * rn.n[0];
     k = divu31(r, rn.div_ny);
     j = r - k * rn.n[1];
 }
@@ -1169,7 +1177,7 @@ __device__ __forceinline__ void yee_b_half_cell(const RunDev &rn, const Fields<R
 {
     const int nx = rn.n[0], ny = rn.n[1], nz = rn.n[2];
     int i, j, k;
-    yee_ijk(rn, (int)l, i, j, k);
+    yee_ijk(rn, l, i, j, k);
     const long long p = rn.cell_base + l;
     const long long pim = p + (i == 0 ? nx - 1 : -1);
     const long long pjm = p + (long long)nx * (j == 0 ? ny - 1 : -1);
@@ -1225,7 +1233,7 @@ __device__ __forceinline__ void yee_e_cell(const RunDev &rn, const Fields<R> &F,
 {
     const int nx = rn.n[0], ny = rn.n[1], nz = rn.n[2];
     int i, j, k;
-    yee_ijk(rn, (int)l, i, j, k);
+    yee_ijk(rn, l, i, j, k);
     const long long p = rn.cell_base + l;
     const long long pip = p + (i == nx - 1 ? -(nx - 1) : 1);
     const long long pjp = p + (long long)nx * (j == ny - 1 ? -(ny - 1) : 1);
@@ -1249,7 +1257,7 @@ __device__ __forceinline__ void yee_b_half_e_cell(const RunDev &rn, const Fields
 {
     const int nx = rn.n[0], ny = rn.n[1], nz = rn.n[2];
     int i, j, k;
-    yee_ijk(rn, (int)l, i, j, k);
+    yee_ijk(rn, l, i, j, k);
     const long long p = rn.cell_base + l;
     const bool f32 = sizeof(R) == 4;
     const R hx = f32 ? R(0.5f * rn.cNf[0]) : R(0.5 * rn.cN[0]), hy = f32 ? R(0.5f * rn.cNf[1]) : R(0.5 * rn.cN[1]);

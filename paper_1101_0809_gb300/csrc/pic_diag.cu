@@ -405,7 +405,7 @@ __global__ void __launch_bounds__(kDiagThreads) k_diag_cells(const RunDev *runs,
     const double id0 = 1.0 / rn.d[0], id1 = 1.0 / rn.d[1], id2 = 1.0 / rn.d[2];
     for (long long l = blockIdx.x * (long long)blockDim.x + threadIdx.x; l < ncell; l += stride) {
         int i, j, k;
-        yee_ijk(rn, (int)l, i, j, k);
+        yee_ijk(rn, l, i, j, k);
         const long long p = rn.cell_base + l;
         const long long pip = p + (i == nx - 1 ? -(nx - 1) : 1), pim = p + (i == 0 ? nx - 1 : -1);
         const long long pjp = p + (long long)nx * (j == ny - 1 ? -(ny - 1) : 1);
