@@ -154,16 +154,18 @@ __device__ __forceinline__ void item_shift(const PartArgs<R> &a, const WorkItem 
     if (threadIdx.x < len) {
         const long long p = it.begin + (len <= NT ? threadIdx.x : len * threadIdx.x / NT);
         const int cell = OLD ? a.old_cell[p] : a.P.cell[p];
-        const int rest = divu31(cell, rn.div_nx);
+        const int at = OLD && cell < 0 ? 0 : cell;   // < 0: none was saved
+        const int rest = divu31(at, rn.div_nx);
         const int k = DIM == 3 ? divu31(rest, rn.div_ny) : 0;
-        const int c[3] = {cell - rest * rn.n[0], rest - k * rn.n[1], k};
+        const int c[3] = {at - rest * rn.n[0], rest - k * rn.n[1], k};
 #pragma unroll
         for (int x = 0; x < DIM; ++x) {
+            if (OLD && cell < 0) break;
             d[x] = 2 * (c[x] - o[x]) - (T[x] - 1);   // twice the distance from the tile's centre, nearest image
             if (d[x] > rn.n[x]) d[x] -= 2 * rn.n[x];
             if (d[x] < -rn.n[x]) d[x] += 2 * rn.n[x];
         }
-        d[3] = 1;
+        d[3] = OLD && cell < 0 ? 0 : 1;
     }
 #pragma unroll
     for (int x = 0; x < 4; ++x) {
@@ -277,6 +279,7 @@ __device__ __noinline__ void far_particle(const PartArgs<R> &a, int group, long 
             }
         } else {
             atomicOr(a.err, ERR_NONFINITE);   // as in process_item: it keeps x^n and contributes no current
+            if (MODE == 1) a.old_cell[p] = -1;
         }
         if (live || RP) {
             if (RP) a.P.id[p] = a.S.id[sp];
@@ -649,7 +652,9 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
     if (PRE) fetch(it.begin + threadIdx.x);
     for (long long pw = it.begin + (threadIdx.x & ~31); pw < it.end; pw += NT) {
         const long long p = pw + lane;
-        const bool valid = p < it.end;
+        bool valid = p < it.end;
+        const int old_cell = MODE == 2 && valid ? a.old_cell[p] : 0;
+        valid = valid && old_cell >= 0;   // < 0: its momentum became non-finite in the push
         const long long pn = pw + NT;   // the warp's next round
         unsigned sp_cur = 0;
         if (RP) {
@@ -670,7 +675,7 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
             // ---- the particle's state at x^n (old) -------------------------------
             const long long sp = RP ? (long long)sp_cur : p;   // where the state is read
             const Pool<R> &src = RP ? a.S : a.P;
-            const int cell0 = PRE ? pre_c : MODE == 2 ? a.old_cell[p] : src.cell[sp];
+            const int cell0 = PRE ? pre_c : MODE == 2 ? old_cell : src.cell[sp];
             o0 = PRE ? pre_o0 : MODE == 2 ? a.old_off[0][p] : src.off[0][sp];
             o1 = PRE ? pre_o1 : MODE == 2 ? a.old_off[1][p] : src.off[1][sp];
             o2 = DIM == 3 ? (PRE ? pre_o2 : MODE == 2 ? a.old_off[2][p] : src.off[2][sp]) : R(0);
@@ -754,6 +759,7 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
                 if (!finite3(w[0], w[1], w[2])) {
                     atomicOr(a.err, ERR_NONFINITE);
                     live = false;   // the particle keeps x^n and contributes no current
+                    if (MODE == 1) a.old_cell[p] = -1;   // (which tells the deposit)
                     if (RP) {   // ... in its slot of the new order, with the momentum it reached
                         a.P.id[p] = PRE ? id : a.S.id[sp];
                         a.P.cell[p] = cell0;
