@@ -122,12 +122,12 @@ cudaError_t launch_step_persistent(int dims, int prec, cudaStream_t st, WorkItem
 // next cell with offset 0.  Momenta are converted; id = index in the call.
 // ---------------------------------------------------------------------------
 // With REC (FP32) the particle is written as one 32-byte record, for the sort's
-// gather.  A position already in [0, N) is taken as it is: the wrap would
+// gather.  A position already in (0, N) is taken as it is: the wrap would
 // subtract N * floor(x / N) = 0, and its FP64 quotient set the kernel's time
 // (16e6 particles: 1.66 ms with it; their 80 bytes each are 0.19 ms of memory).
 __device__ __forceinline__ double wrap_position(double x, double N)
 {
-    if (x >= 0.0 && x < N) return x;
+    if (x > 0.0 && x < N) return x;   // (-0.0 becomes 0.0 below)
     x -= N * floor(x / N);
     if (x >= N) x -= N;
     if (x < 0.0) x = 0.0;
