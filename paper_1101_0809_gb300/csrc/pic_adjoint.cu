@@ -405,15 +405,19 @@ __device__ __forceinline__ void adj_particle(const AdjArgs<R> &a, const GroupDev
             e[ax] = hq * Ep[ax];
             t[ax] = w0[ax] + e[ax];
         }
-        const R rg = R(1) / sqrt(t[0] * t[0] + t[1] * t[1] + t[2] * t[2] + c2);
-        const R s = hq * rg;
+        const R gt = sqrt(t[0] * t[0] + t[1] * t[1] + t[2] * t[2] + c2);
+        // FP32: two reciprocals instead of the five quotients that FP64 keeps, each of
+        // which it would round once more
+        constexpr bool F64 = sizeof(R) == 8;
+        const R rg = R(1) / gt;
+        const R s = F64 ? hq / gt : hq * rg;
         #pragma unroll
         for (int ax = 0; ax < 3; ++ax) b[ax] = s * Bp[ax];
         nn3[0] = t[0] + (t[1] * b[2] - t[2] * b[1]);
         nn3[1] = t[1] + (t[2] * b[0] - t[0] * b[2]);
         nn3[2] = t[2] + (t[0] * b[1] - t[1] * b[0]);
         const R b2 = b[0] * b[0] + b[1] * b[1] + b[2] * b[2];
-        const R rb = R(1) / (R(1) + b2);
+        const R d2 = R(1) + b2, rb = R(1) / d2;
         const R Fq = R(2) * rb;
         m[0] = nn3[1] * b[2] - nn3[2] * b[1];
         m[1] = nn3[2] * b[0] - nn3[0] * b[2];
@@ -434,7 +438,7 @@ __device__ __forceinline__ void adj_particle(const AdjArgs<R> &a, const GroupDev
         lb[0] = lm[1] * nn3[2] - lm[2] * nn3[1];
         lb[1] = lm[2] * nn3[0] - lm[0] * nn3[2];
         lb[2] = lm[0] * nn3[1] - lm[1] * nn3[0];
-        const R lb2 = lF * (-R(2) * rb * rb);
+        const R lb2 = lF * (F64 ? -R(2) / (d2 * d2) : -R(2) * rb * rb);
         #pragma unroll
         for (int ax = 0; ax < 3; ++ax) lb[ax] += R(2) * b[ax] * lb2;
         // n = t + t x b: lt += ln + b x ln, lb += ln x t
@@ -450,10 +454,10 @@ __device__ __forceinline__ void adj_particle(const AdjArgs<R> &a, const GroupDev
             ls += lb[ax] * Bp[ax];
             lBp[ax] = s * lb[ax];
         }
-        const R lgt = -ls * s * rg;
+        const R lgt = F64 ? -ls * hq / (gt * gt) : -ls * s * rg;
         #pragma unroll
         for (int ax = 0; ax < 3; ++ax) {
-            lt[ax] += lgt * t[ax] * rg;
+            lt[ax] += F64 ? lgt * t[ax] / gt : lgt * t[ax] * rg;
             lw0[ax] = lt[ax];
             lEp[ax] = hq * (le[ax] + lt[ax]);
         }

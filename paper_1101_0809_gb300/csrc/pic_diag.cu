@@ -400,9 +400,6 @@ __global__ void __launch_bounds__(kDiagThreads) k_diag_cells(const RunDev *runs,
     const long long ncell = (long long)nx * ny * nz;
     const long long stride = (long long)gridDim.x * blockDim.x;
     const double hx = 0.5 * rn.cN[0], hy = 0.5 * rn.cN[1], hz = 0.5 * rn.cN[2];
-    // the FP64 pipe bounds this kernel: reciprocals of the cell sizes instead of three
-    // quotients per cell
-    const double id0 = 1.0 / rn.d[0], id1 = 1.0 / rn.d[1], id2 = 1.0 / rn.d[2];
     for (long long l = blockIdx.x * (long long)blockDim.x + threadIdx.x; l < ncell; l += stride) {
         int i, j, k;
         yee_ijk(rn, l, i, j, k);
@@ -411,14 +408,14 @@ __global__ void __launch_bounds__(kDiagThreads) k_diag_cells(const RunDev *runs,
         const long long pjp = p + (long long)nx * (j == ny - 1 ? -(ny - 1) : 1);
         const long long pjm = p + (long long)nx * (j == 0 ? ny - 1 : -1);
         const double ex = F.E[0][p], ey = F.E[1][p], ez = F.E[2][p];
-        double div = ((double)F.E[0][pip] - ex) * id0 + ((double)F.E[1][pjp] - ey) * id1;
+        double div = ((double)F.E[0][pip] - ex) / rn.d[0] + ((double)F.E[1][pjp] - ey) / rn.d[1];
         double bx = (double)F.B[0][p] - hy * (ez - (double)F.E[2][pjm]);
         double by = (double)F.B[1][p] + hx * (ez - (double)F.E[2][pim]);
         double bz = (double)F.B[2][p] - hx * (ey - (double)F.E[1][pim]) + hy * (ex - (double)F.E[0][pjm]);
         if (DIM == 3) {
             const long long pkp = p + (long long)nx * ny * (k == nz - 1 ? -(nz - 1) : 1);
             const long long pkm = p + (long long)nx * ny * (k == 0 ? nz - 1 : -1);
-            div += ((double)F.E[2][pkp] - ez) * id2;
+            div += ((double)F.E[2][pkp] - ez) / rn.d[2];
             bx += hz * (ey - (double)F.E[1][pkm]);
             by -= hz * (ex - (double)F.E[0][pkm]);
         }
