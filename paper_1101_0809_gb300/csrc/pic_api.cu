@@ -185,7 +185,7 @@ cudaError_t alloc_pool(pic_grid *g, PoolBuf &P, long long n)
     if (n == 0) return cudaSuccess;
     auto part = [](size_t bytes) { return (bytes + 255) & ~(size_t)255; };   // cudaMalloc's own alignment
     const size_t wi = part(n * sizeof(int)), wr = part(n * elem(g));
-    const size_t bytes = std::max(2 * wi + (g->dims + 3) * wr, (size_t)n * sizeof(LoadRec));
+    const size_t bytes = 2 * wi + (g->dims + 3) * wr;
     const cudaError_t e = dalloc_bytes(&P.slab, bytes);
     if (e != cudaSuccess) return e;
     P.bytes = bytes;
@@ -453,7 +453,7 @@ int do_sort(pic_grid *g, bool defer = false, bool rec = false)
                                          g->sort_order == PIC_SORT_CELL_LANES ? g->lane_count : nullptr,
                                          g->tiles_valid && g->sort_order != PIC_SORT_CELL_LANES ? 1 : 0,
                                          defer ? &perm : nullptr,
-                                         rec ? static_cast<const LoadRec *>(g->pool_alt.slab) : nullptr);
+                                         rec ? g->pool_alt.slab : nullptr);
     launch_count_add(g, nl);
     g->tiles_valid = false;
     if (e != cudaSuccess) return cuda_fail(e, "tile sort");
@@ -1106,8 +1106,7 @@ static int load_many(pic_grid *g, std::vector<LoadReq> &reqs, int on_device)
         const RunDev &rn = g->runs[q.run].dev;
         launch_count_add(g, 1);
         return launch_load(g->prec, g->stream, q.n, src[r][0], src[r][1], src[r][2], src[r][3], src[r][4], src[r][5],
-                           g->dims, rn.n[0], rn.n[1], rn.n[2], P, base,
-                           rec ? static_cast<LoadRec *>(alt.slab) : nullptr);
+                           g->dims, rn.n[0], rn.n[1], rn.n[2], P, base, rec ? alt.slab : nullptr);
     };
     // every request matches a loaded group of the same size: convert in place
     bool in_place = true;
@@ -1130,8 +1129,8 @@ static int load_many(pic_grid *g, std::vector<LoadReq> &reqs, int on_device)
                 bool stays = h.n > 0;
                 for (auto *m : match) stays = stays && m != &h;
                 if (!stays) continue;
-                CK(launch_copy_pool_rec(g->stream, g->pool, h.base, g->pool.cell,
-                                        static_cast<LoadRec *>(g->pool_alt.slab), h.base, h.n, g->dims),
+                CK(launch_copy_pool_rec(g->stream, g->pool, h.base, g->pool.cell, g->pool_alt.slab, h.base, h.n,
+                                        g->dims),
                    "particle load");
                 launch_count_add(g, 1);
             }
@@ -1183,8 +1182,7 @@ static int load_many(pic_grid *g, std::vector<LoadReq> &reqs, int on_device)
         if (e != cudaSuccess) break;
         if (h.base >= 0) {   // an old group keeps its data
             if (h.n > 0) {
-                e = rec ? launch_copy_pool_rec(g->stream, g->pool, h.base, np.cell, static_cast<LoadRec *>(na.slab),
-                                               pb, h.n, g->dims)
+                e = rec ? launch_copy_pool_rec(g->stream, g->pool, h.base, np.cell, na.slab, pb, h.n, g->dims)
                         : launch_copy_pool(g->prec, g->stream, g->pool, h.base, np, pb, h.n);
                 launch_count_add(g, 1);
             }

@@ -31,7 +31,7 @@ struct HostGroup {
 // Device buffers of a particle pool (one of two, swapped by the sort), all parts
 // of one allocation.
 struct PoolBuf {
-    void *slab = nullptr;   // the allocation: >= sizeof(LoadRec) per particle in FP32
+    void *slab = nullptr;   // the allocation: >= sizeof(LoadRec<dims>) per particle in FP32
     size_t bytes = 0;
     int *cell = nullptr;
     void *off[3] = {nullptr, nullptr, nullptr};
@@ -81,18 +81,28 @@ cudaError_t launch_step_persistent(int dims, int prec, cudaStream_t st, WorkItem
                                    const unsigned *perm = nullptr);
 cudaError_t particles_set_smem_limit(int dims, int prec, int mode, size_t bytes, int order2 = 3);
 
-// An FP32 particle as the load hands it to the sort: one 32-byte sector, so that
-// the sort's gather reads one sector per particle whatever the input order.
-struct __align__(16) LoadRec {
+// An FP32 particle as the load hands it to the sort, so that the sort's gather
+// reads few sectors per particle whatever the input order: one in 3D, one or two in
+// 2D, where a record is as long as a pool's particle and no longer.
+template <int DIM>
+struct LoadRec;
+template <>
+struct __align__(16) LoadRec<3> {
     int cell, id;
     float off[3], w[3];
 };
+template <>
+struct LoadRec<2> {
+    int cell, id;
+    float off[2], w[3];
+};
+static_assert(sizeof(LoadRec<3>) == 32 && sizeof(LoadRec<2>) == 28, "a pool's bytes per particle");
 
-// rec != nullptr (FP32): LoadRec p goes to rec[base + p] and its cell to P.cell
-// (for the sort's keys); the other arrays of P are not written.
+// rec != nullptr (FP32): record p goes to rec[base + p] (LoadRec<dims>) and its cell
+// to P.cell (for the sort's keys); the other arrays of P are not written.
 cudaError_t launch_load(int prec, cudaStream_t st, long long n, const double *x0, const double *x1,
                         const double *x2, const double *w0, const double *w1, const double *w2,
-                        int dims, int nx, int ny, int nz, const PoolBuf &P, long long base, LoadRec *rec = nullptr);
+                        int dims, int nx, int ny, int nz, const PoolBuf &P, long long base, void *rec = nullptr);
 
 cudaError_t launch_yee(int prec, int which, int zero_j, cudaStream_t st, const RunDev *runs, int nruns,
                        long long max_cells, void *const E[3], void *const B[3], void *const J[3], int dims,
@@ -108,7 +118,7 @@ cudaError_t launch_antenna_tick(cudaStream_t st, long long *ant_n, int nruns);
 cudaError_t launch_copy_pool(int prec, cudaStream_t st, const PoolBuf &src, long long src_base,
                              const PoolBuf &dst, long long dst_base, long long n);
 // The same from an FP32 pool into records (and dst_cell).
-cudaError_t launch_copy_pool_rec(cudaStream_t st, const PoolBuf &src, long long src_base, int *dst_cell, LoadRec *rec,
+cudaError_t launch_copy_pool_rec(cudaStream_t st, const PoolBuf &src, long long src_base, int *dst_cell, void *rec,
                                  long long dst_base, long long n, int dims);
 
 // Sort: computes keys, sorts them stably, permutes the pool from `src` into
@@ -142,7 +152,7 @@ cudaError_t sort_and_build_items(int prec, int dims, cudaStream_t st, long long 
                                  long long *tile_start, unsigned *item_scan, WorkItem *items, int *n_items,
                                  int particles_per_item, int halo, int banked, int half, int *launches,
                                  unsigned char *lane_cell = nullptr, int *lane_count = nullptr, int resort = 0,
-                                 const unsigned **perm_out = nullptr, const LoadRec *rec = nullptr);
+                                 const unsigned **perm_out = nullptr, const void *rec = nullptr);
 // With lane_cell and lane_count (total_tiles * 128 entries each) the order
 // inside a tile is the cell-lane order (PIC_SORT_CELL_LANES) instead of the
 // banked or stable one, and the two tables receive every tile's lane cells
@@ -153,7 +163,7 @@ cudaError_t sort_and_build_items(int prec, int dims, cudaStream_t st, long long 
 // are not moved: *perm_out receives the permutation (dst[o] = src[perm[o]], in
 // the sort scratch, valid until the next sort) for the caller to apply.  With rec
 // (FP32, a full sort, not for the cell-lane order or l_a = 2 1/2) the particles
-// are the records rec[0 .. total) and src holds their cells only; dst may be src.
+// are the records (LoadRec<dims>) rec[0 .. total) and src holds their cells only; dst may be src.
 cudaError_t launch_permute(int prec, int dims, cudaStream_t st, long long total, const PoolBuf &src,
                            const PoolBuf &dst, const unsigned *perm);
 

@@ -121,7 +121,7 @@ cudaError_t launch_step_persistent(int dims, int prec, cudaStream_t st, WorkItem
 // precision, periodic wrap into [0, N); an offset that rounds to 1 moves to the
 // next cell with offset 0.  Momenta are converted; id = index in the call.
 // ---------------------------------------------------------------------------
-// With REC (FP32) the particle is written as one 32-byte record, for the sort's
+// With REC (FP32) the particle is written as one record (LoadRec), for the sort's
 // gather.  A position already in (0, N) is taken as it is: the wrap would
 // subtract N * floor(x / N) = 0, and its FP64 quotient set the kernel's time
 // (16e6 particles: 1.66 ms with it; their 80 bytes each are 0.19 ms of memory).
@@ -134,9 +134,21 @@ __device__ __forceinline__ double wrap_position(double x, double N)
     return x;
 }
 
+template <int DIM>
+__device__ __forceinline__ void put_record(void *rec, long long q, int cell, int id, const float of[3], const float w[3])
+{
+    if constexpr (DIM == 3) {
+        int4 *r = reinterpret_cast<int4 *>(static_cast<LoadRec<3> *>(rec) + q);
+        r[0] = make_int4(cell, id, __float_as_int(of[0]), __float_as_int(of[1]));
+        reinterpret_cast<float4 *>(r)[1] = make_float4(of[2], w[0], w[1], w[2]);
+    } else {
+        static_cast<LoadRec<2> *>(rec)[q] = {cell, id, {of[0], of[1]}, {w[0], w[1], w[2]}};
+    }
+}
+
 template <typename R, int DIM, bool REC>
 __global__ void k_load(long long n, const double *x0, const double *x1, const double *x2, const double *w0,
-                       const double *w1, const double *w2, int nx, int ny, int nz, PoolBuf P, LoadRec *rec,
+                       const double *w1, const double *w2, int nx, int ny, int nz, PoolBuf P, void *rec,
                        long long base)
 {
     const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -162,9 +174,8 @@ __global__ void k_load(long long n, const double *x0, const double *x1, const do
     const int cell = ci[0] + nx * (ci[1] + ny * ci[2]);
     P.cell[base + p] = cell;
     if constexpr (REC) {
-        int4 *r = reinterpret_cast<int4 *>(rec + base + p);
-        r[0] = make_int4(cell, (int)p, __float_as_int(of[0]), __float_as_int(of[1]));
-        reinterpret_cast<float4 *>(r)[1] = make_float4(of[2], (float)ws[0], (float)ws[1], (float)ws[2]);
+        const float w[3] = {(float)ws[0], (float)ws[1], (float)ws[2]};
+        put_record<DIM>(rec, base + p, cell, (int)p, of, w);
     } else {
 #pragma unroll
         for (int a = 0; a < DIM; ++a) static_cast<R *>(P.off[a])[base + p] = of[a];
@@ -177,7 +188,7 @@ __global__ void k_load(long long n, const double *x0, const double *x1, const do
 template <int DIM>
 static void load_t(int prec, cudaStream_t st, unsigned nb, int nt, long long n, const double *x0, const double *x1,
                    const double *x2, const double *w0, const double *w1, const double *w2, int nx, int ny, int nz,
-                   const PoolBuf &P, LoadRec *rec, long long base)
+                   const PoolBuf &P, void *rec, long long base)
 {
     if (prec == 0)
         k_load<double, DIM, false><<<nb, nt, 0, st>>>(n, x0, x1, x2, w0, w1, w2, nx, ny, nz, P, nullptr, base);
@@ -189,7 +200,7 @@ static void load_t(int prec, cudaStream_t st, unsigned nb, int nt, long long n, 
 
 cudaError_t launch_load(int prec, cudaStream_t st, long long n, const double *x0, const double *x1,
                         const double *x2, const double *w0, const double *w1, const double *w2, int dims, int nx,
-                        int ny, int nz, const PoolBuf &P, long long base, LoadRec *rec)
+                        int ny, int nz, const PoolBuf &P, long long base, void *rec)
 {
     if (n <= 0) return cudaSuccess;
     const int nt = 256;
@@ -203,19 +214,19 @@ cudaError_t launch_load(int prec, cudaStream_t st, long long n, const double *x0
 
 // A range of an FP32 pool into records, for a load that keeps other groups.
 template <int DIM>
-__global__ void k_copy_pool_rec(long long n, PoolBuf S, long long sb, int *cell, LoadRec *rec, long long db)
+__global__ void k_copy_pool_rec(long long n, PoolBuf S, long long sb, int *cell, void *rec, long long db)
 {
     const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (p >= n) return;
     auto at = [&](void *v) { return static_cast<const float *>(v)[sb + p]; };
     const int c = S.cell[sb + p];
     if (cell + db != S.cell + sb) cell[db + p] = c;
-    int4 *r = reinterpret_cast<int4 *>(rec + db + p);
-    r[0] = make_int4(c, S.id[sb + p], __float_as_int(at(S.off[0])), __float_as_int(at(S.off[1])));
-    reinterpret_cast<float4 *>(r)[1] = make_float4(DIM == 3 ? at(S.off[2]) : 0.f, at(S.w[0]), at(S.w[1]), at(S.w[2]));
+    const float of[3] = {at(S.off[0]), at(S.off[1]), DIM == 3 ? at(S.off[2]) : 0.f};
+    const float w[3] = {at(S.w[0]), at(S.w[1]), at(S.w[2])};
+    put_record<DIM>(rec, db + p, c, S.id[sb + p], of, w);
 }
 
-cudaError_t launch_copy_pool_rec(cudaStream_t st, const PoolBuf &src, long long sb, int *dst_cell, LoadRec *rec,
+cudaError_t launch_copy_pool_rec(cudaStream_t st, const PoolBuf &src, long long sb, int *dst_cell, void *rec,
                                  long long db, long long n, int dims)
 {
     if (n <= 0) return cudaSuccess;

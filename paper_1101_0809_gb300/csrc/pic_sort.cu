@@ -1201,37 +1201,31 @@ static cudaError_t launch_permute4(int prec, int dims, cudaStream_t st, long lon
 }
 
 // The gather of a load: slot q of the arrays takes record perm[q].  Bound by
-// memory: 36 bytes read and 32 written per particle, the read a whole sector.
+// memory: in 3D 36 bytes read and 32 written per particle, the read a whole sector.
 // Four slots per thread, a block apart, keep as many sectors in flight while the
 // writes stay coalesced.
 constexpr int kRecSlots = 4;
 template <int DIM>
-__global__ void __launch_bounds__(256) k_permute_rec(long long total, const unsigned *perm, const LoadRec *rec,
+__global__ void __launch_bounds__(256) k_permute_rec(long long total, const unsigned *perm, const LoadRec<DIM> *rec,
                                                      PoolBuf dst)
 {
     const long long q0 = blockIdx.x * (long long)(kRecSlots * 256) + threadIdx.x;
-    int4 a[kRecSlots];
-    float4 b[kRecSlots];
+    LoadRec<DIM> a[kRecSlots];
 #pragma unroll
     for (int s = 0; s < kRecSlots; ++s) {
         const long long q = q0 + s * 256;
-        if (q >= total) continue;
-        const int4 *r = reinterpret_cast<const int4 *>(rec + perm[q]);
-        a[s] = r[0];
-        b[s] = reinterpret_cast<const float4 *>(r)[1];
+        if (q < total) a[s] = rec[perm[q]];
     }
 #pragma unroll
     for (int s = 0; s < kRecSlots; ++s) {
         const long long q = q0 + s * 256;
         if (q >= total) continue;
-        dst.cell[q] = a[s].x;
-        dst.id[q] = a[s].y;
-        static_cast<float *>(dst.off[0])[q] = __int_as_float(a[s].z);
-        static_cast<float *>(dst.off[1])[q] = __int_as_float(a[s].w);
-        if (DIM == 3) static_cast<float *>(dst.off[2])[q] = b[s].x;
-        static_cast<float *>(dst.w[0])[q] = b[s].y;
-        static_cast<float *>(dst.w[1])[q] = b[s].z;
-        static_cast<float *>(dst.w[2])[q] = b[s].w;
+        dst.cell[q] = a[s].cell;
+        dst.id[q] = a[s].id;
+#pragma unroll
+        for (int c = 0; c < DIM; ++c) static_cast<float *>(dst.off[c])[q] = a[s].off[c];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) static_cast<float *>(dst.w[c])[q] = a[s].w[c];
     }
 }
 
@@ -1247,7 +1241,7 @@ cudaError_t sort_and_build_items(int prec, int dims, cudaStream_t st, long long 
                                  long long *tile_start, unsigned *item_scan, WorkItem *items, int *n_items,
                                  int particles_per_item, int halo, int banked, int half, int *launches,
                                  unsigned char *lane_cell, int *lane_count, int resort, const unsigned **perm_out,
-                                 const LoadRec *rec)
+                                 const void *rec)
 {
     if (lane_cell) perm_out = nullptr;
     if (rec && (prec == 0 || lane_cell || half || resort || perm_out)) return cudaErrorInvalidValue;
@@ -1397,9 +1391,9 @@ cudaError_t sort_and_build_items(int prec, int dims, cudaStream_t st, long long 
     if (rec) {
         const unsigned nbr = (unsigned)((total + kRecSlots * nt - 1) / (kRecSlots * nt));
         if (dims == 3)
-            k_permute_rec<3><<<nbr, nt, 0, st>>>(total, scr.vals[cur], rec, dst);
+            k_permute_rec<3><<<nbr, nt, 0, st>>>(total, scr.vals[cur], static_cast<const LoadRec<3> *>(rec), dst);
         else
-            k_permute_rec<2><<<nbr, nt, 0, st>>>(total, scr.vals[cur], rec, dst);
+            k_permute_rec<2><<<nbr, nt, 0, st>>>(total, scr.vals[cur], static_cast<const LoadRec<2> *>(rec), dst);
         *launches += 1;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         return build_items(st, tile_start, total_tiles, particles_per_item, groups, ngroups, scr, item_scan, items,

@@ -91,3 +91,24 @@ def test_sorts_ends_and_snapshots_between_the_places(P, dims, interval, ppc):
             assert float(np.abs(u[order] - v[ob]).max()) <= steps * 64 * 2.0 ** -52 * float(np.abs(v).max())
     for g in (a, b, c, d):
         g.close()
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("dims", [2, 3])
+def test_memory_of_the_particles(P, prec, dims):
+    import torch
+    n = (256, 256, 1) if dims == 2 else (64, 64, 64)
+    count = 6_000_000
+    x = [torch.rand(count, dtype=torch.float64, device="cuda") * n[a] for a in range(3)]
+    w = [torch.zeros(count, dtype=torch.float64, device="cuda") for _ in range(3)]
+    took = None
+    for again in range(2):                # the first time brings the library's one-time allocations
+        g = P.Grid(P.make_desc(dims, n, (1.0,) * 3, 0.02, 20.0, prec))
+        before = used()
+        P.pic_load_particles(g.h, 0, -1.0, 1.0, 1.0, x, w)
+        took = used() - before
+        g.close()
+    es = 8 if prec == 0 else 4
+    # two pools of cell, id, offsets and momenta; keys and values twice and a class byte
+    # for the sort; the old cell and offsets; 20 MiB for the tables and page rounding
+    assert took <= count * (2 * (8 + es * (dims + 3)) + 17 + 4 + es * dims) + (20 << 20)
