@@ -85,6 +85,13 @@ struct WorkItem {
     int drifted;          // particles found past the staged tile, summed over the steps since the sort
 };
 
+// The sum of WorkItem::drifted with one step's count, held at the largest int: an
+// item may go unsorted for any number of steps.
+__host__ __device__ __forceinline__ int add_drifted(int sum, int more)
+{
+    return more > 0x7fffffff - sum ? 0x7fffffff : sum + more;
+}
+
 template <typename R>
 struct Pool {
     int *cell;

@@ -927,7 +927,7 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
         }
         if (MODE != 2 && threadIdx.x == 0) {   // the sort policy's measure of drift, and item_shift's
             atomicAdd(reinterpret_cast<unsigned *>(a.err) + 1, (unsigned)nf_all);
-            a.items[item].drifted = it.drifted + nf_all;
+            a.items[item].drifted = add_drifted(it.drifted, nf_all);
         }
     }
     if (NEED_J) {

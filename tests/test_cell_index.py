@@ -53,3 +53,26 @@ def host_run(tmp_path, source):
 def test_cell_indices_below_and_above_two_to_the_31(tmp_path):
     done, bad = map(int, host_run(tmp_path, SOURCE))
     assert done > 1_000_000 and bad == 0
+
+
+DRIFT = r"""
+#include <cstdio>
+#include "pic_device.cuh"
+int main()
+{
+    const int most = 0x7fffffff;
+    int sum = 0, bad = 0;
+    for (long long step = 1; step <= 300000; ++step) {   // 8192 particles a step pass 2^31 after 262144
+        sum = pic::add_drifted(sum, 8192);
+        const long long want = 8192 * step;
+        bad += sum != (want < most ? (int)want : most);
+    }
+    bad += pic::add_drifted(most, 0) != most || pic::add_drifted(0, most) != most || pic::add_drifted(3, 4) != 7;
+    printf("%d\n", bad);
+    return 0;
+}
+"""
+
+
+def test_drift_sums_stay_at_the_largest_int(tmp_path):
+    assert host_run(tmp_path, DRIFT) == ["0"]
