@@ -6,6 +6,8 @@
 //   rest mass, B^n = B^{n-1/2} - (1/2) c curl_h E^n), and the momentum sum.
 // Sums are per-block tree reductions written to fixed slots and reduced by one
 // block in slot order.
+#include <type_traits>
+
 #include "pic_internal.h"
 
 namespace pic {
@@ -388,6 +390,14 @@ __global__ void __launch_bounds__(kDiagThreads, 4) k_diag_items(int run, const W
     block_reduce_store(v, -1, partials + (long long)blockIdx.x * kPartVals);
 }
 
+// Whether d > 0 is a power of two with a normal reciprocal.
+__device__ __forceinline__ bool power_of_two(double d)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(d);
+    const int e = (int)(b >> 52);
+    return (b & ((1ull << 52) - 1)) == 0 && e > 0 && e < 2046;
+}
+
 // Cells: residual against the reference, charge, field energies.
 // Partial slots: 0 max |r - r_ref|, 1 sum (r - r_ref)^2, 2 charge, 3 sum E^2, 4 sum B^2.
 template <int DIM, typename R>
@@ -400,35 +410,46 @@ __global__ void __launch_bounds__(kDiagThreads) k_diag_cells(const RunDev *runs,
     const long long ncell = (long long)nx * ny * nz;
     const long long stride = (long long)gridDim.x * blockDim.x;
     const double hx = 0.5 * rn.cN[0], hy = 0.5 * rn.cN[1], hz = 0.5 * rn.cN[2];
-    for (long long l = blockIdx.x * (long long)blockDim.x + threadIdx.x; l < ncell; l += stride) {
-        int i, j, k;
-        yee_ijk(rn, l, i, j, k);
-        const long long p = rn.cell_base + l;
-        const long long pip = p + (i == nx - 1 ? -(nx - 1) : 1), pim = p + (i == 0 ? nx - 1 : -1);
-        const long long pjp = p + (long long)nx * (j == ny - 1 ? -(ny - 1) : 1);
-        const long long pjm = p + (long long)nx * (j == 0 ? ny - 1 : -1);
-        const double ex = F.E[0][p], ey = F.E[1][p], ez = F.E[2][p];
-        double div = ((double)F.E[0][pip] - ex) / rn.d[0] + ((double)F.E[1][pjp] - ey) / rn.d[1];
-        double bx = (double)F.B[0][p] - hy * (ez - (double)F.E[2][pjm]);
-        double by = (double)F.B[1][p] + hx * (ez - (double)F.E[2][pim]);
-        double bz = (double)F.B[2][p] - hx * (ey - (double)F.E[1][pim]) + hy * (ex - (double)F.E[0][pjm]);
-        if (DIM == 3) {
-            const long long pkp = p + (long long)nx * ny * (k == nz - 1 ? -(nz - 1) : 1);
-            const long long pkm = p + (long long)nx * ny * (k == 0 ? nz - 1 : -1);
-            div += ((double)F.E[2][pkp] - ez) / rn.d[2];
-            bx += hz * (ey - (double)F.E[1][pkm]);
-            by -= hz * (ex - (double)F.E[0][pkm]);
+    // FP64 instructions bound this kernel, three quotients by the cell sizes above all
+    // (96^3 cells: 0.04 ms).  By a power of two the product with the reciprocal is the
+    // quotient, to the last bit; only then is it taken.
+    const double id0 = 1.0 / rn.d[0], id1 = 1.0 / rn.d[1], id2 = 1.0 / rn.d[2];
+    auto cells = [&](auto p2) {
+        auto over = [&](double a, double d, double id) { return p2 ? a * id : a / d; };
+        for (long long l = blockIdx.x * (long long)blockDim.x + threadIdx.x; l < ncell; l += stride) {
+            int i, j, k;
+            yee_ijk(rn, l, i, j, k);
+            const long long p = rn.cell_base + l;
+            const long long pip = p + (i == nx - 1 ? -(nx - 1) : 1), pim = p + (i == 0 ? nx - 1 : -1);
+            const long long pjp = p + (long long)nx * (j == ny - 1 ? -(ny - 1) : 1);
+            const long long pjm = p + (long long)nx * (j == 0 ? ny - 1 : -1);
+            const double ex = F.E[0][p], ey = F.E[1][p], ez = F.E[2][p];
+            double div = over((double)F.E[0][pip] - ex, rn.d[0], id0) + over((double)F.E[1][pjp] - ey, rn.d[1], id1);
+            double bx = (double)F.B[0][p] - hy * (ez - (double)F.E[2][pjm]);
+            double by = (double)F.B[1][p] + hx * (ez - (double)F.E[2][pim]);
+            double bz = (double)F.B[2][p] - hx * (ey - (double)F.E[1][pim]) + hy * (ex - (double)F.E[0][pjm]);
+            if (DIM == 3) {
+                const long long pkp = p + (long long)nx * ny * (k == nz - 1 ? -(nz - 1) : 1);
+                const long long pkm = p + (long long)nx * ny * (k == 0 ? nz - 1 : -1);
+                div += over((double)F.E[2][pkp] - ez, rn.d[2], id2);
+                bx += hz * (ey - (double)F.E[1][pkm]);
+                by -= hz * (ex - (double)F.E[0][pkm]);
+            }
+            const double rt = rho[p] + rn.rho_bg;
+            const double res = div - 4.0 * kPi * rt;
+            if (set_ref) ref[p] = res;
+            const double dr = res - ref[p];
+            v[0] = fmax(v[0], fabs(dr));
+            v[1] += dr * dr;
+            v[2] += rt * rn.V;
+            v[3] += ex * ex + ey * ey + ez * ez;
+            v[4] += bx * bx + by * by + bz * bz;
         }
-        const double rt = rho[p] + rn.rho_bg;
-        const double res = div - 4.0 * kPi * rt;
-        if (set_ref) ref[p] = res;
-        const double dr = res - ref[p];
-        v[0] = fmax(v[0], fabs(dr));
-        v[1] += dr * dr;
-        v[2] += rt * rn.V;
-        v[3] += ex * ex + ey * ey + ez * ez;
-        v[4] += bx * bx + by * by + bz * bz;
-    }
+    };
+    if (power_of_two(rn.d[0]) && power_of_two(rn.d[1]) && power_of_two(rn.d[2]))
+        cells(std::true_type());
+    else
+        cells(std::false_type());
     block_reduce_store(v, 0, partials + (long long)blockIdx.x * kPartVals);
 }
 

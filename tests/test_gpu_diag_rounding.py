@@ -18,7 +18,8 @@ def P():
 
 
 @pytest.mark.parametrize("prec", [0, 1])
-@pytest.mark.parametrize("dims,n,d", [(2, (19, 14, 1), (0.3, 0.7, 1.0)), (3, (13, 15, 11), (0.3, 0.7, 1.1))])
+@pytest.mark.parametrize("dims,n,d", [(2, (19, 14, 1), (0.3, 0.7, 1.0)), (3, (13, 15, 11), (0.3, 0.7, 1.1)),
+                                      (3, (13, 15, 11), (0.5, 2.0, 1.0)), (2, (19, 14, 1), (0.25, 0.7, 1.0))])
 def test_residual_is_the_divergence_of_e(P, prec, dims, n, d):
     g = P.Grid(P.make_desc(dims, n, d, 0.01, 9.0, prec, tile=(4, 4, 4), halo=0))
     rng = np.random.Generator(np.random.PCG64(88))
