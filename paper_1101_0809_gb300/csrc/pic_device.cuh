@@ -34,9 +34,22 @@ inline DivU31 make_divu31(int d)
     v.L = L;
     return v;
 }
-__host__ __device__ __forceinline__ int divu31(int n, const DivU31 &v)
+__device__ __forceinline__ int divu31(int n, const DivU31 &v)
 {
     return (int)(((unsigned long long)(unsigned)n * v.m) >> v.L);
+}
+
+// l / d for cell numbers, with inv = ceil(2^64 / d), d >= 2: l inv / 2^64 exceeds the
+// quotient by less than l / 2^64, and by less than 1/d while l d < 2^64 (fewer than
+// 2^33 cells fit the device, d < 2^31).
+inline unsigned long long make_inv(int d) { return ~0ull / (unsigned)d + 1; }
+__host__ __device__ __forceinline__ long long div_cells(long long l, unsigned long long inv)
+{
+#ifdef __CUDA_ARCH__
+    return (long long)__umul64hi((unsigned long long)l, inv);
+#else
+    return (long long)((unsigned __int128)(unsigned long long)l * inv >> 64);
+#endif
 }
 
 struct RunDev {
@@ -57,6 +70,7 @@ struct RunDev {
     double fpdt;            // 4 pi dt
     float fpdtf;            // 4 pi dt in FP32
     DivU31 div_nx, div_ny;  // division by n[0] and n[1]
+    unsigned long long inv_nx, inv_ny;  // the same of cell numbers from 2^31 on (div_cells)
     DivU31 div_t[3];        // division by the tile extents
     float cf, cNf[3];     // c and the Courant numbers in FP32
 };
@@ -1139,23 +1153,16 @@ __device__ __forceinline__ double antenna_field(const RunDev &rn, double x, doub
 __device__ __forceinline__ double add_incident(double v, double k, double f) { return fma(k, f, v); }
 __device__ __forceinline__ float add_incident(float v, double k, double f) { return v + (float)(k * f); }
 
-// The cell indices of cell l of a run.  Without 64-bit quotients below 2^31, where
-// they set the Yee kernels' time (256x64x64 cells FP32: 20.9 us per B half step and
-// 24.0 us per E step, 48 and 60 bytes per cell); a run without particles may
-// have more cells.
+// The cell indices of cell l of a run.  Without quotients, which set the Yee kernels'
+// time (256x64x64 cells FP32: 20.9 us per B half step and 24.0 us per E step, 48 and
+// 60 bytes per cell), and in 64 bits, since a run without particles may have 2^31
+// cells and more.
 __host__ __device__ __forceinline__ void yee_ijk(const RunDev &rn, long long l, int &i, int &j, int &k)
 {
-    if (l >> 31 != 0) {
-        const long long r = l / rn.n[0];
-        i = (int)(l - r * rn.n[0]);
-        k = (int)(r / rn.n[1]);
-        j = (int)(r - (long long)k * rn.n[1]);
-        return;
-    }
-    const int r = divu31((int)l, rn.div_nx);
-    i = (int)l - r * rn.n[0];
-    k = divu31(r, rn.div_ny);
-    j = r - k * rn.n[1];
+    const long long r = div_cells(l, rn.inv_nx);
+    i = (int)(l - r * rn.n[0]);
+    k = (int)div_cells(r, rn.inv_ny);
+    j = (int)(r - (long long)k * rn.n[1]);
 }
 
 // The B half step's new values at a cell, h = c dt/(2 d): the fused multiply-adds

@@ -14,13 +14,13 @@ SOURCE = r"""
 using namespace pic;
 int main()
 {
-    const int sizes[][3] = {{1290, 1290, 1291}, {65537, 65536, 1}, {3, 1, 1 << 30}, {7, 5, 3}, {2147483647, 1, 3}};
+    const int sizes[][3] = {{1290, 1290, 1291}, {65537, 65536, 1}, {5, 5, 1 << 28}, {7, 5, 9}, {1073741827, 7, 1}, {8, 1 << 30, 1}};
     long long bad = 0, done = 0;
     for (auto &n : sizes) {
         RunDev rn{};
         for (int a = 0; a < 3; ++a) rn.n[a] = n[a];
-        rn.div_nx = make_divu31(n[0]);
-        rn.div_ny = make_divu31(n[1]);
+        rn.inv_nx = make_inv(n[0]);
+        rn.inv_ny = make_inv(n[1]);
         const long long cells = (long long)n[0] * n[1] * n[2], edge = 1LL << 31;
         for (long long at : {0LL, cells / 2, edge - 70000, edge - 3, edge, 2 * edge - 3, cells - 70000, cells - 3})
             for (long long l = at < 0 ? 0 : at; l < cells && l < at + 70000; ++l) {
