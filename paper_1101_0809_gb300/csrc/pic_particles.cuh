@@ -652,9 +652,7 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
     if (PRE) fetch(it.begin + threadIdx.x);
     for (long long pw = it.begin + (threadIdx.x & ~31); pw < it.end; pw += NT) {
         const long long p = pw + lane;
-        bool valid = p < it.end;
-        const int old_cell = MODE == 2 && valid ? a.old_cell[p] : 0;
-        valid = valid && old_cell >= 0;   // < 0: its momentum became non-finite in the push
+        const bool valid = p < it.end;
         const long long pn = pw + NT;   // the warp's next round
         unsigned sp_cur = 0;
         if (RP) {
@@ -675,7 +673,7 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
             // ---- the particle's state at x^n (old) -------------------------------
             const long long sp = RP ? (long long)sp_cur : p;   // where the state is read
             const Pool<R> &src = RP ? a.S : a.P;
-            const int cell0 = PRE ? pre_c : MODE == 2 ? old_cell : src.cell[sp];
+            const int cell0 = PRE ? pre_c : MODE == 2 ? a.old_cell[p] : src.cell[sp];
             o0 = PRE ? pre_o0 : MODE == 2 ? a.old_off[0][p] : src.off[0][sp];
             o1 = PRE ? pre_o1 : MODE == 2 ? a.old_off[1][p] : src.off[1][sp];
             o2 = DIM == 3 ? (PRE ? pre_o2 : MODE == 2 ? a.old_off[2][p] : src.off[2][sp]) : R(0);
@@ -705,10 +703,11 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
             lk = DIM == 3 ? local_coord(k, oz, T2, G, nz) : 0;
             const bool inr =
                 li >= -G && li < T0 + G && lj >= -G && lj < T1 + G && (DIM == 2 || (lk >= -G && lk < T2 + G));
-            far = !inr;
+            const bool saved = MODE != 2 || cell0 >= 0;   // < 0: its momentum became non-finite in the push
+            far = !inr && saved;
 
             n0 = o0; n1 = o1; n2 = o2;
-            live = inr;
+            live = inr && saved;
             if (far) {
                 // stepped later, with 31 others
             } else if (MODE != 2) {
