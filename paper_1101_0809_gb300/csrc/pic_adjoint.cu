@@ -405,12 +405,15 @@ __device__ __forceinline__ void adj_particle(const AdjArgs<R> &a, const GroupDev
             e[ax] = hq * Ep[ax];
             t[ax] = w0[ax] + e[ax];
         }
-        const R gt = sqrt(t[0] * t[0] + t[1] * t[1] + t[2] * t[2] + c2);
-        // FP32: two reciprocals instead of the five quotients that FP64 keeps, each of
-        // which it would round once more
+        // Two reciprocals instead of five quotients.  In FP64 as precise: with CUDA's
+        // rsqrt (pic_device.cuh) each product has as many roundings as the quotient it
+        // stands for, but for 2/(1 + b.b)^2, which stays one.  In FP32 the error of the
+        // whole pass against 64 bits was measured, and did not grow.
         constexpr bool F64 = sizeof(R) == 8;
-        const R rg = R(1) / gt;
-        const R s = F64 ? hq / gt : hq * rg;
+        const R g2 = t[0] * t[0] + t[1] * t[1] + t[2] * t[2] + c2;
+        R rg;
+        if constexpr (F64) rg = rsqrt(g2); else rg = R(1) / sqrt(g2);
+        const R s = hq * rg;
         #pragma unroll
         for (int ax = 0; ax < 3; ++ax) b[ax] = s * Bp[ax];
         nn3[0] = t[0] + (t[1] * b[2] - t[2] * b[1]);
@@ -454,10 +457,10 @@ __device__ __forceinline__ void adj_particle(const AdjArgs<R> &a, const GroupDev
             ls += lb[ax] * Bp[ax];
             lBp[ax] = s * lb[ax];
         }
-        const R lgt = F64 ? -ls * hq / (gt * gt) : -ls * s * rg;
+        const R lgt = -ls * s * rg;
         #pragma unroll
         for (int ax = 0; ax < 3; ++ax) {
-            lt[ax] += F64 ? lgt * t[ax] / gt : lgt * t[ax] * rg;
+            lt[ax] += lgt * t[ax] * rg;
             lw0[ax] = lt[ax];
             lEp[ax] = hq * (le[ax] + lt[ax]);
         }
