@@ -191,12 +191,21 @@ struct GlobalZeroB5 {   // offsets -2..2 from the l_a = 2 1/2 base index
 // ORD = 5 (l_a = 2 1/2): E and rho tiles with a halo of (halo + 2) cells, the
 // 4-cell cubic weights around the base index.  ORD = 4 (Eq. wrong1): the same
 // halo for its gather, the l_a = 1 1/2 charge.
-// Four blocks per SM, at the price of spills (96^3 cells of 8 + 8 particles: a step
-// pass with diagnostics 5.48 ms, 5.52 at three blocks, about 5.6 at two without spills).
+// Blocks per SM: four, at the price of spills, but for the 3D ones of Eq. wrong1.  A
+// call at two / three / four blocks: 2D, 512x512 cells of 16 + 16 particles, 322 / 273 /
+// 250 us; 3D, 64^3 of 16 + 16, l_a = 2 1/2 815 / 779 / 744 us, Eq. wrong1 569 / 497 / 506
+// and with 8x8x8 tiles 619 / 545 / 593, l_a = 1 1/2 470 / 421 / 432; the last stay at four
+// for smaller items (96^3 of 8 + 8 particles, 4 steps and a call: 5.57 ms at three, 5.54
+// at four; 64^3 of 2 + 2 the same).
+template <int DIM, int ORD>
+constexpr int diag_blocks()
+{
+    return DIM == 3 && ORD == 4 ? 3 : 4;
+}
 template <int DIM, int ORD = 3>
-__global__ void __launch_bounds__(kDiagThreads, 4) k_diag_items(int run, const WorkItem *items, const int *n_items,
-                                                             const GroupDev *groups, const RunDev *runs, Pool<float> P,
-                                                             Fields<float> F, int halo, double *rho, double *partials)
+__global__ void __launch_bounds__(kDiagThreads, diag_blocks<DIM, ORD>())
+    k_diag_items(int run, const WorkItem *items, const int *n_items, const GroupDev *groups, const RunDev *runs,
+                 Pool<float> P, Fields<float> F, int halo, double *rho, double *partials)
 {
     extern __shared__ __align__(16) unsigned char dsm[];
     double v[kPartVals] = {0, 0, 0, 0, 0, 0, 0, 0};

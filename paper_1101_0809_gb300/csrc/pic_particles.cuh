@@ -58,19 +58,26 @@ constexpr int kQueueVals = 7;
 // 3D FP64: room for both kinds of particles that moved, fewer than 32 of each and 32 new
 constexpr int kQueueCap3 = 96;
 
-// Blocks per SM the kernels are compiled for: two (128 registers), three of the
-// 2D FP32 ones (80).  Where the shared tiles leave room for one block only, the
-// launches take the variant compiled for one.  In FP32 that has 512 threads, to
-// have as many warps as two blocks would (61x47x53 cells in 8x8x8 tiles, 12 + 12
-// particles each, 20 steps: 7.76 ms with 256 threads and all registers, 6.54 with
-// 512).  In FP64 it has 256 threads whose registers hold everything: every 3D tile
-// spilled 100 to 200 bytes per thread at 128 registers (48^3 cells, 16 + 16
-// particles each: 5.3 -> 4.7 ms a step).  The 2D FP32 persistent step of 24 runs took 22.5 ms per 30 steps at
-// two blocks, 19.7 at three and 21.0 at four.
-template <int DIM, typename R>
+// Blocks per SM the kernels are compiled for: two (128 registers); three of the 2D
+// FP32 fused step (80); four of the 2D FP32 split calls (64), whose 512 items of
+// 256x256 cells and 16 + 16 particles then run at once (the push 40 us, 47 at three;
+// the deposit 55 us, 64 at three and 61 at five).  Where the shared tiles leave room
+// for one block only, the launches take the variant compiled for one.  In FP32 that
+// has 512 threads, to have as many warps as two blocks would; in FP64 it has 256
+// threads whose registers hold everything, where every 3D tile spilled 100 to 200
+// bytes per thread at 128.
+template <int DIM, typename R, int MODE>
 constexpr int min_blocks()
 {
-    return DIM == 2 && sizeof(R) == 4 ? 3 : 2;
+    return DIM == 2 && sizeof(R) == 4 ? (MODE == 0 ? 3 : 4) : 2;
+}
+// ... of the persistent step: the compiled geometries as the fused step (24 runs, 30
+// steps: 18.1 ms, 19.5 at two), tiles read at run time at two (384x384 cells of 16 + 16
+// particles, 10 steps: 12x12 tiles 1.75 ms, 1.79 at three; 24x24 1.83, 2.11 at three).
+template <int DIM, typename R, bool DYN>
+constexpr int min_blocks_persistent()
+{
+    return DYN ? 2 : min_blocks<DIM, R, 0>();
 }
 template <typename R, bool ONE>
 constexpr int block_threads()
@@ -709,7 +716,7 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
             n0 = o0; n1 = o1; n2 = o2;
             live = inr && saved;
             if (far) {
-                // stepped later, with 31 others
+                // stepped after the others, a block's width of them at a time
             } else if (MODE != 2) {
                 R Ep[3], Bp[3];
                 if constexpr (ORD == 5) {
@@ -1118,7 +1125,7 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
 }
 
 template <int DIM, typename R, int MODE, class GEO = GeoDyn, int ORD = 3, bool PERM = false, bool ONE = false>
-__global__ void __launch_bounds__(block_threads<R, ONE>(), ONE ? 1 : min_blocks<DIM, R>())
+__global__ void __launch_bounds__(block_threads<R, ONE>(), ONE ? 1 : min_blocks<DIM, R, MODE>())
     k_particles(const __grid_constant__ PartArgs<R> a)
 {
     if ((int)blockIdx.x >= *a.n_items) return;
@@ -1143,7 +1150,7 @@ __device__ __forceinline__ int find_run(const long long *run_cell_base, int nrun
 // PERM: the step right after a sort that left the arrays in place; the work
 // items read the particles through the permutation (as k_particles does).
 template <int DIM, typename R, class GEO = GeoDyn, bool PERM = false, bool ONE = false>
-__global__ void __launch_bounds__(kThreads, ONE ? 1 : min_blocks<DIM, R>()) k_step_persistent(const __grid_constant__ PartArgs<R> a, int nruns,
+__global__ void __launch_bounds__(kThreads, ONE ? 1 : min_blocks_persistent<DIM, R, GEO::dyn>()) k_step_persistent(const __grid_constant__ PartArgs<R> a, int nruns,
                                                               const long long *run_cell_base, long long *ant_n,
                                                               int antennas)
 {
