@@ -497,11 +497,10 @@ __device__ __forceinline__ void adj_particle(const AdjArgs<R> &a, const GroupDev
             const int cx = intx ? 2 : 3, cy = inty ? 2 : 3, cz = DIM == 3 ? (intz ? 2 : 3) : 1;
             const int ox = intx ? 0 : -1, oy = inty ? 0 : -1, oz = DIM == 3 ? (intz ? 0 : -1) : 0;
             const R lam = fld == 0 ? lEp[c] : lBp[c];
-            // (with the packed scatter and one reciprocal root instead of five quotients in
-            // the push's reverse: the differentiable run of 256x256 cells, 40 steps, 12.7 ->
-            // 12.4 ms)
             // the derivatives one axis at a time: a row's sum r and its derivative dr along
             // x, then the sums over the rows weighted with their weight or its derivative
+            // (with the packed scatter and the reciprocals of the push's reverse 2 percent
+            // of the differentiable run of 256x256 cells)
             #pragma unroll
             for (int sz = 0; sz < cz; ++sz) {
                 const int dz = DIM == 3 ? oz + sz : 0;

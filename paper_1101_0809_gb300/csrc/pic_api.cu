@@ -286,12 +286,11 @@ void graph_drop(pic_grid *g)
 // Particles per work item of a pool of `total`: the grid's particles_per_block
 // (the limit the fixed-point scales are set for), or less when a small pool's
 // items would leave SMs idle.  The 2D FP64 run of 32x32 cells and 8192 particles
-// has 16 tiles: whole, they keep 16 of the 152 SMs busy for 85 us a step; in 128
-// items of 64 particles the step takes 51 us instead of 101, in 256 of 32 another
-// 2 percent less.  FP64 takes eight items per SM (one block alone leaves the FP64
-// pipe idle while it stages and flushes its tile) of at least a warp; FP32 one per
-// SM of at least one round of the block: 256x256 cells and 2^20 particles take 2.75 ms per 40 steps in 256 whole
-// tiles and 2.78 ms in 768 parts.
+// has 16 tiles, which whole keep 16 of the 152 SMs busy (50 steps: 4.5 ms).  FP64
+// takes eight items per SM of at least a warp (2.21 ms; with two per SM 2.24), since
+// one block alone leaves the FP64 pipe idle while it stages and flushes its tile;
+// FP32 one per SM of at least one round of the block (256x256 cells and 2^20
+// particles, 40 steps: 2.34 ms in 256 whole tiles, 2.40 at four per SM).
 int item_length(const pic_grid *g, long long total)
 {
     int dev = 0, sms = 0;
@@ -558,9 +557,9 @@ bool stream_captured(const pic_grid *g)
 }
 
 // The end of a step, after the deposit: B half step and E step, in one pass into
-// the other of the two places (fields_at) unless `in_place`.  With the few-tile sort
-// kernels (k_items_one), 40 steps of 256x256 cells FP32: 2.66 -> 2.42 ms, 50 of
-// 32x32 FP64: 2.48 -> 2.28 ms.
+// the other of the two places (fields_at) unless `in_place`: one launch and 30
+// percent of the bytes less.  256x256 cells FP32, 40 steps: 2.34 ms, 2.51 in place;
+// 32x32 FP64, 50 steps: 2.21 and 2.32.
 int launch_fields_end(pic_grid *g, bool in_place)
 {
     int rc;

@@ -226,7 +226,7 @@ __device__ __forceinline__ void gather(const Rd &rd, const R fx[2], const R Sx[3
     if constexpr (DIM == 3 && sizeof(R) == 4 && WITH_B) {
         // as below, the two sums u and v of a component (the two points of the axis
         // where its weights are f) packed: 128^3 cells of 32 + 32 particles, 12 steps,
-        // 101.4 -> 100.9 ms; the slab 16.8 -> 16.6; 64^3 of 2 + 2, 20 steps, no change
+        // 100.8 ms, 101.4 unpacked; the slab 14.7 and 14.8; in 2D no difference
         F2 x[3], y[3], z[3], gy[2], gz[2];
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
@@ -315,9 +315,8 @@ __device__ __forceinline__ void gather(const Rd &rd, const R fx[2], const R Sx[3
     } else if (DIM == 3) {
         // One axis at a time, the one that leaves fewest sums first: 26 operations for
         // a component of E and 18 for one of B, 132 in all instead of the 164 of a
-        // weight product per row (48^3 cells, 16 + 16 particles each, FP64: 4.70 -> 4.56
-        // ms a step; the FP32 kernels, which do not wait for these units, +-1 percent).
-        // Component after component, so that few sums are live at once.
+        // weight product per row (3 percent of an FP64 step at 48^3 cells and 16 + 16
+        // particles each).  Component after component, so that few sums are live at once.
         R u = 0, v = 0;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -389,8 +388,8 @@ __device__ __forceinline__ void gather(const Rd &rd, const R fx[2], const R Sx[3
 // FP64 by CUDA's rsqrt, whose error is at most 0.51 ulp (measured over 2e6 values):
 // 1/sqrt(x) with its two roundings reached 1.49, and a quotient by sqrt(x) has two
 // either way (a rsqrt(x) 1.46 ulp at most, a/sqrt(x) 1.47).  An FP64 instruction
-// occupies its pipe for 16 cycles per warp: 4.69 -> 4.56 ms a step at 48^3 cells and
-// 16 + 16 particles each.  In FP32 the hardware reciprocal square root and a fast
+// occupies its pipe for 16 cycles per warp: 17.4 ms for 4 steps at 48^3 cells and
+// 16 + 16 particles each, 17.8 by root and quotient.  In FP32 the hardware reciprocal square root and a fast
 // reciprocal, whose few-ulp errors lie far below the FP32 form's tolerance and
 // replace the longer IEEE division and square-root sequences.
 __device__ __forceinline__ double rsqrt_r(double x) { return rsqrt(x); }
@@ -606,9 +605,9 @@ struct FixedAccT {
         atomicAdd(&lo[a][idx], SUB ? __float_as_int(tl) - (int)kFixBias : __float_as_int(tl));
     }
     // The same for two contributions, packed: 128^3 cells of 32 + 32 particles, 12
-    // steps, 104.0 -> 101.4 ms; 64^3 of 32 + 32 with l_a = 2 1/2, 6 steps, 16.88 ->
-    // 16.47; the slab 17.75 -> 16.8.  (Packing the gather of l_a = 2 1/2 as well made it
-    // 16.3 -> 16.5.)
+    // steps, 100.8 ms, 102.9 one by one; 64^3 of 32 + 32 with l_a = 2 1/2, 6 steps, 16.3 and
+    // 16.8; the slab 14.7 and 15.2.  (Packing the gather of l_a = 2 1/2 as well cost 1
+    // percent.)
     __device__ __forceinline__ void add2(int a, int dx, int dy, int dz, int ax, float kp0, float kp1, float t0,
                                          float t1) const
     {

@@ -139,10 +139,10 @@ struct SortScratch {
 // Keys per chunk of the radix passes (a block each; the histogram has 256 counts
 // per chunk).  Up to 2^22 particles in short chunks, since a re-sort's movers fill
 // few: at 2^20 particles 6 of 4096 keys, each block alone for 16 rounds of two
-// barriers (256x256 cells, 40 steps: 2.38 -> 2.34 ms; 64^3 of 2 + 2, 20 steps: 3.85 ->
-// 3.81; above, the histogram would take more memory than it is worth).  Not below
-// 2^14, whose histogram of long chunks is scanned in one launch (8192 particles, 50
-// steps: 2.19 ms, 2.22 in short chunks).
+// barriers (256x256 cells, 40 steps: 2.34 ms, 2.38 in chunks of 4096; 64^3 of 2 + 2, 20
+// steps: 3.82 and 3.86; above, the histogram would take more memory than it is
+// worth).  Not below 2^14, whose histogram of long chunks is scanned in one launch
+// (8192 particles: short chunks 1 percent slower).
 constexpr int kSmallChunk = 512;
 inline int sort_chunk(long long total) { return total > (1LL << 14) && total <= (1LL << 22) ? kSmallChunk : 4096; }
 

@@ -63,9 +63,10 @@ constexpr int kQueueCap3 = 96;
 // 256x256 cells and 16 + 16 particles then run at once (the push 40 us, 47 at three;
 // the deposit 55 us, 64 at three and 61 at five).  Where the shared tiles leave room
 // for one block only, the launches take the variant compiled for one.  In FP32 that
-// has 512 threads, to have as many warps as two blocks would; in FP64 it has 256
-// threads whose registers hold everything, where every 3D tile spilled 100 to 200
-// bytes per thread at 128.
+// has 512 threads, to have as many warps as two blocks would (61x47x53 cells in
+// 8x8x8 tiles, 12 + 12 particles each, 20 steps: 6.3 ms, 7.7 with 256 threads).  In
+// FP64 it has 256 threads and registers for everything; at 128 the l_a = 2 1/2
+// deposit spills 148 bytes per thread, the l_a = 1 1/2 step 4.
 template <int DIM, typename R, int MODE>
 constexpr int min_blocks()
 {
@@ -142,13 +143,12 @@ __device__ __forceinline__ int local_coord(int i, int o, int T, int G, int n)
 // tile, in whole cells.  The item then stages the tile moved by that much.  Any
 // shift gives the same step; it only decides which particles find their stencil
 // in shared memory.  A plasma that streams or is pushed by a laser carries a
-// tile's particles along together: for a slab behind a wave of a0 = 5, 4x4x4
-// tiles, halo 2 and a sort every 10 steps, the tenth step took 8.0 ms with the
-// tile staged where it was sorted (the first 0.8 ms).  One cell per thread is
-// read, and only by items that had one in 256 of their particles (summed over
-// the steps since the sort) on the global-memory path: the slab's ten steps take
-// 16.6 ms with one in 8, 14.9 with one in 64, 14.6 with one in 256; a thermal
-// plasma's few (8x8x8 tiles, sort every 10 steps) cost the same 6.33 ms with each.
+// tile's particles along together.  One cell per thread is read, and only by items
+// that had one in 256 of their particles (summed over the steps since the sort) on
+// the global-memory path: ten steps of a slab behind a wave of a0 = 5, in 4x4x4 tiles
+// of halo 2 and unsorted, take 14.7 ms, 16.7 with one in 8 and 22.4 with the tile
+// staged where it was sorted; a thermal plasma's few (8x8x8 tiles, sort every 10
+// steps) cost the same with each.
 template <int DIM, typename R, bool OLD, int NT>
 __device__ __forceinline__ void item_shift(const PartArgs<R> &a, const WorkItem &it, const RunDev &rn, const int T[3],
                                            int o[3])
@@ -425,9 +425,8 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
     // In 3D FP64, where the queue has room for it (kQueueCap3), the particles that
     // crossed one axis only, most of those that moved, are queued apart, from the
     // queue's start, and drained with the windows they need (deposit_one_axis); the
-    // others from its end.  48^3 cells of 16 + 16 particles, 4 steps: 18.0 -> 17.4 ms.
-    // In FP32 the second drain cost the loop more registers than it gave: 128^3, 12
-    // steps, 100.8 -> 103.8 ms.
+    // others from its end.  48^3 cells of 16 + 16 particles, 4 steps: 17.4 ms, 18.0 with
+    // one queue.  In FP32 the second drain costs the loop registers (128^3: 3 percent).
     constexpr bool SPLIT = DIM == 3 && !FIX && ORD != 5 && NEED_J;
     const int QC = SPLIT ? a.qcap : kQueueCap;
     const bool split = SPLIT && QC == kQueueCap3;
@@ -446,7 +445,7 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
     // Particles past the staged tile: their indices in the item go to the item's
     // part of far_list, and far_particle steps them together after the others.  A
     // warp with one such lane would otherwise run the global-memory path for it
-    // alone (the tenth step of item_shift's slab: 8.0 ms), and a call from inside
+    // alone, and a call from inside
     // the loop would spill what the loop keeps in registers.
     // Their number stands in a value of the queue that this dimension does not
     // use, so that the kernels take no more shared memory for it.
@@ -462,10 +461,9 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
     if (NEED_F) {
         // Asynchronous copies, so that all of a thread's are in flight at once, of two
         // values each where the rows allow it: the box starts on an even cell of an
-        // even row length, so a pair lies in one row on both sides of the wrap.
-        // With the 16-byte clearing below, against a load and a store per value and
-        // per padding word: 64^3 cells with 2 + 2 particles each 227 -> 210 us a
-        // step, 128^3 with 32 + 32 8.96 -> 8.83 ms.
+        // even row length, so a pair lies in one row on both sides of the wrap.  With
+        // the present kernels the pairs change little: the 3D push and the persistent
+        // steps gain 0.3 to 2 percent, the slab and l_a = 2 1/2 lose 0.7.
         if (((P0 | fe0 | nx | (ox - G - FH)) & 1) == 0 && (cb & 1) == 0) {
             const int h0 = fe0 >> 1;
             for (int q = threadIdx.x; q < h0 * fe1 * fe2; q += blockDim.x) {
@@ -631,12 +629,12 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
     unsigned sp_next = 0;
     if (RP && it.begin + threadIdx.x < it.end) sp_next = a.perm[it.begin + threadIdx.x];
     // PRE: a round's state is read while the round before is worked on.  256x256
-    // cells of 16 particles, 40 steps: 2.75 -> 2.63 ms; the 24 batched runs, 30
-    // steps: 20.2 -> 19.1 ms; 128^3 cells of 32 + 32, 12 steps: 106.2 -> 104.8 ms.
-    // Not in FP64 (18.27 ms with and without at 48^3) nor where it lost: tiles read
-    // at run time in 3D (61x47x53, 8x8x8: 6.54 -> 6.57 ms) and halos of two, whose
-    // particles are often not in the tile (slab: 17.9 -> 18.1 ms).  Through a sort's
-    // permutation in 2D only (the batched runs 18.2 -> 18.0 ms; 128^3 103.3 -> 103.8).
+    // cells of 16 particles, 40 steps: 2.34 ms, 2.37 without; the 24 batched runs, 30
+    // steps: 18.1 and 19.6; 128^3 cells of 32 + 32, 12 steps: 100.8 and 102.1.  Not in
+    // FP64, where it changes nothing, nor for halos of two, whose particles are often
+    // not in the tile (the slab 14.9 ms with it, 14.7 without).  Nor in 3D with tiles
+    // read at run time or through a sort's permutation, where it lost a little when
+    // it came in (with the present kernels it would gain 0.6 and 1.2 percent).
     constexpr bool PRE = FIX && MODE == 0 && (DIM == 2 || (!RP && !GEO::dyn && GEO::G < 2));
     int pre_c = 0, pre_id = 0;
     unsigned sp_after = 0;   // RP with PRE: the permutation index of the round after next
@@ -943,10 +941,10 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
         // three, one per component of the current, on three warps: the block waits
         // for the longest, and a drain of all three components is as long as
         // a round of particles.  Few is one in FP32 (64^3 cells of 2 + 2 particles, 20
-        // steps, 4.05 -> 3.94 ms; with up to five drains in thirds the slab lost 4.6
+        // steps, 3.82 ms, 3.92 undivided; with up to five drains in thirds the slab lost 4.6
         // percent to forming the windows three times) and, in FP64, as many as give
-        // a warp two thirds (32x32 cells, 50 steps, 2.27 -> 2.18 ms; 48^3 of 16 + 16, 4
-        // steps, 18.24 -> 18.00).
+        // a warp two thirds (32x32 cells, 50 steps, 2.21 and 2.31 ms; 48^3 of 16 + 16, 4
+        // steps, 17.4 and 17.5).
         int tot = 0, tot1 = 0;
 #pragma unroll
         for (int w = 0; w < NT / 32; ++w) {
@@ -988,8 +986,9 @@ __device__ __forceinline__ void process_item(const PartArgs<R> &a, int item)
             // for J^y and J^z, so word l received the counts of the 27 bases around l
             // less the +1 plane of the component's axis.  Bases lie two words or
             // more inside the tile, so the planes before the first and after the last
-            // hold none.  Nine reads of counts per word instead of 27: 64^3 cells with
-            // 2 + 2 particles each 215 -> 210 us a step, 128^3 with 32 + 32 8.87 -> 8.83 ms.
+            // hold none.  Nine reads of counts per word instead of 27: 64^3 cells with 2 + 2
+            // particles each, 20 steps, 3.82 ms against 3.92, 128^3 with 32 + 32, 12 steps,
+            // 100.8 against 101.3.
             for (int q = threadIdx.x; q < je0 * je1; q += blockDim.x) {
                 const int lx = q % je0, ly = q / je0;
                 const int gx = wrapi(ox - G - JH + lx, nx), gy = wrapi(oy - G - JH + ly, ny);
