@@ -34,6 +34,10 @@
  *     pic_deposit_current, pic_yee_update and pic_sort return without waiting.
  *     Device-side failures (a non-finite momentum) are latched in an error word
  *     that pic_sync and pic_diagnostics read and report as PIC_ERR_NONFINITE.
+ *   - the caller may capture pic_step (without the adaptive sort policy),
+ *     pic_gather_push, pic_deposit_current and pic_yee_update on the grid's stream.
+ *     Such a graph stays valid until a load or a sort moves the particles: between
+ *     calls E, B and J keep their device addresses for the grid's life.
  */
 #ifndef PIC_H
 #define PIC_H
